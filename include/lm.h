@@ -284,6 +284,14 @@ lm_status lm_mdot_backward(lm_solver *solver, const void *forces, const void *to
  *   Single-wall solvers: threads 128 or 256, ilp 1, 2, 4 (scalar) or 2, 4
  *   (packed = 1); FP64 ilp 1.  All forms give results within the FP32
  *   tolerance of the FP64 product; they differ in rounding order only.
+ *   These are the one-sided kernels, which evaluate every ordered pair.  Where
+ *   the symmetric kernel (every unordered pair once; no configuration of its
+ *   own) is faster, a solver uses it instead: LM_FP64 in the open geometry, and
+ *   from N = 3000 LM_FP32C without angular blocks or above a wall.  Its results
+ *   are bitwise reproducible too, and its partial sums take up to 128 slots of
+ *   3 or 6 FP64 values per particle (or 256 MiB if that is more); when they do
+ *   not fit, the one-sided kernel runs.  lm_set_pair_config pins the one-sided
+ *   kernel for the solver; lm_autotune tunes it without pinning it.
  */
 /* Launch configuration of the pair kernels (no paper counterpart):
  *   threads: CTA size and j-tile length (128 or 256);

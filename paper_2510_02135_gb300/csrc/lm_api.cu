@@ -172,7 +172,11 @@ struct lm_solver {
 
     lm_pair_config cfg{128, 4, 1, 0};
     bool cfg_forced = false;
+    bool cfg_pinned = false;   // set by lm_set_pair_config: that one-sided kernel, never the symmetric form
     int64_t cfg_N = -1;
+    lmk::SymPlan sym{};        // symmetric form of the product, planned for sym_N particles
+    bool sym_ok = false;
+    int64_t sym_N = -1;
     lm_pair_config adj_cfg{128, 1, 1, 0};
     int64_t adj_cfg_N = -1;
 
@@ -425,8 +429,27 @@ void ensure_config(lm_solver* s) {
     s->cfg_N = s->N;
 }
 
+// Whether the product takes the symmetric form: its rule selects this (precision,
+// blocks, geometry, N), no one-sided kernel is pinned and its partial sums fit
+// the device (else the one-sided form, which needs fewer, serves).
+bool sym_form(lm_solver* s) {
+    if (s->cfg_pinned) return false;
+    if (s->sym_N != s->N) {
+        s->sym_ok = lmk::sym_plan(s->fp64, s->angular, s->wall, s->N, s->sm_count, &s->sym);
+        s->sym_N = s->N;
+    }
+    if (!s->sym_ok) return false;
+    const size_t bytes =
+        (size_t)s->sym.slots * lmk::mdot_partial_components(s->angular) * (size_t)s->N * sizeof(double);
+    if (s->partials.ensure(bytes) != cudaSuccess) {
+        cudaGetLastError();
+        s->sym_ok = false;
+    }
+    return s->sym_ok;
+}
+
 lm_status run_mdot(lm_solver* s, const void* F, const void* T, int in_f64, void* lin, void* ang, int out_f64,
-                   const lm_pair_config& cfg, const void* pos4_override = nullptr) {
+                   const lm_pair_config& cfg, const void* pos4_override = nullptr, bool one_sided = false) {
     lmk::MdotArgs a;
     a.fp64 = s->fp64;
     a.angular = s->angular;
@@ -445,8 +468,11 @@ lm_status run_mdot(lm_solver* s, const void* F, const void* T, int in_f64, void*
     a.splits = cfg.splits;
     a.packed = cfg.packed;
     a.partials = nullptr;
+    const bool sym = !one_sided && sym_form(s);
     const int64_t se = lmk::mdot_effective_splits(s->N, cfg.threads, cfg.splits);
-    if (se > 1) {
+    if (sym) {
+        a.partials = s->partials.as<double>();
+    } else if (se > 1) {
         const size_t bytes =
             (size_t)se * lmk::mdot_partial_components(s->angular) * (size_t)s->N * sizeof(double);
         LM_CUDA(s->partials.ensure(bytes), "allocating split partial sums");
@@ -463,7 +489,9 @@ lm_status run_mdot(lm_solver* s, const void* F, const void* T, int in_f64, void*
         s->prof_used += 1;
         s->prof_pairs += (double)s->N * (double)s->N;
     }
-    if (s->wall)
+    if (sym)
+        LM_CUDA(lmk::launch_sym_mdot(a, s->sym, s->wall, s->stream), "symmetric mobility product kernel");
+    else if (s->wall)
         LM_CUDA(lmk::launch_wall_mdot(a, s->stream), "mobility product kernel (single wall)");
     else
         LM_CUDA(lmk::launch_mdot(a, s->stream), "mobility product kernel");
@@ -1362,6 +1390,7 @@ lm_status lm_set_pair_config(lm_solver* s, const lm_pair_config* cfg) {
         s->cfg.splits = s->has_pos ? auto_splits(s->N, cfg->threads, cfg->ilp, occ * s->sm_count) : 1;
     }
     s->cfg_forced = true;
+    s->cfg_pinned = true;
     s->cfg_N = s->has_pos ? s->N : -1;
     return LM_OK;
 }
@@ -1452,7 +1481,8 @@ lm_status autotune_impl(lm_solver* s, int reps, lm_pair_config* best) {
     };
     lm_pair_config best_cfg = default_config(s, N);
     lm_status result = pick(
-        [&](const lm_pair_config& c) { return run_mdot(s, fin, fin + bytes, s->fp64, fout, fout + bytes, s->fp64, c); },
+        [&](const lm_pair_config& c) { return run_mdot(s, fin, fin + bytes, s->fp64, fout, fout + bytes, s->fp64, c,
+                                                    nullptr, true); },
         cands, &best_cfg);
     // the packed translation adjoint (open geometry): threads x ilp x j per vote x splits
     if (result == LM_OK && !s->fp64 && !s->angular && !s->wall) {

@@ -197,6 +197,17 @@ cudaError_t launch_mdot(const MdotArgs& a, cudaStream_t s);
 bool wall_config_supported(int fp64, int threads, int ilp, int packed);
 int wall_ctas_per_sm(int fp64, int angular, int threads, int ilp, int packed);
 cudaError_t launch_wall_mdot(const MdotArgs& a, cudaStream_t s);
+// Symmetric form of the product (sym_kernels.cu): every unordered pair once.
+// slots * (3 or 6) * N doubles of partial sums.
+struct SymPlan {
+    int threads, ilp, tile;       // CTA size, i-particles per thread, particles per j-tile
+    int64_t tb, T;                // j-tiles per i-block, j-tiles
+    int64_t m, nsuper, chunk;     // i-blocks per superblock, superblocks, j-tiles per item
+    int64_t slots;
+};
+// The plan for a product that the symmetric form serves best, else false.
+bool sym_plan(int fp64, int angular, int wall, int64_t N, int sm_count, SymPlan* p);
+cudaError_t launch_sym_mdot(const MdotArgs& a, const SymPlan& p, int wall, cudaStream_t s);
 cudaError_t launch_adjoint(const AdjointArgs& a, cudaStream_t s);
 int adjoint_partial_components(int angular);
 int adjoint_ilp(int fp64, int angular);

@@ -20,6 +20,18 @@ template <> struct V4<double> { using type = lmk::dvec4; };
 __device__ __forceinline__ float rsq(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double rsq(double x) { return 1.0 / sqrt(x); }
 
+// 1 / sqrt(x) for normal x > 0 in the far field.  FP64: the instruction's
+// estimate (relative error d, 2^-20 or better) and one third-order step,
+// y (1 + e (1/2 + 3 e / 8)) with e = 1 - x y^2, which leaves (5/2) d^3 and the
+// rounding: 5 FP64 operations against about 20 for 1 / sqrt.
+__device__ __forceinline__ float rsq_far(float x) { return rsqrtf(x); }
+__device__ __forceinline__ double rsq_far(double x) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-(x * y), y, 1.0);
+    return fma(fma(0.375, e, 0.5), e * y, y);
+}
+
 template <typename R>
 __device__ __forceinline__ R load_elem(const void* p, int in_f64, int64_t idx) {
     if (p == nullptr) return R(0);

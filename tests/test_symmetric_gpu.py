@@ -1,0 +1,97 @@
+"""The symmetric product (every unordered pair once, both particles written)
+against the FP64 oracle at the sizes where its blocks, tiles, item rows and
+superblocks change, against the pinned one-sided kernel, and bitwise against
+itself."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from paper_2510_02135_gb300 import lm  # noqa: E402
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    from paper_2510_02135_gb300 import _build
+
+    _build.build()
+
+
+def dev(x):
+    return None if x is None else torch.from_numpy(np.ascontiguousarray(x)).cuda()
+
+
+def rel(y, ref):
+    y, ref = np.asarray(y, np.float64).ravel(), np.asarray(ref, np.float64).ravel()
+    return np.linalg.norm(y - ref) / np.linalg.norm(ref)
+
+
+def system(n, dt, wall):
+    """Spheres at volume fraction about 0.1 with overlapping neighbours, a
+    coincident pair whose members lie in different blocks, and above a wall
+    some particles that touch or cross it."""
+    rng = np.random.default_rng(n)
+    side = (n * 42.0) ** (1.0 / 3.0) + 1.0
+    pos = rng.uniform(-side / 2, side / 2, (n, 3))
+    if wall:
+        pos[:, 2] = rng.uniform(-0.3, side, n)
+    if n > 2:
+        pos[n - 1] = pos[0]
+        pos[n // 2] = pos[1] + [0.9, 0.2, 0.3]
+    F, T = rng.standard_normal((2, n, 3))
+    return pos.astype(dt), F.astype(dt), T.astype(dt)
+
+
+# FP64: i-blocks of 128, j-tiles of 32.  FP32: j-tiles of 128, i-blocks of 256
+# (free space up to N = 10000, wall), 512 (to 40000) and 1024; from N = 131073
+# blocks are joined into superblocks so that the slots stay at 128.
+CASES = ([(n, ang, True, False) for n in (1, 2, 33, 128, 129, 1000) for ang in (False, True)]
+         + [(n, False, False, False) for n in (3000, 3329, 10001, 40001, 150001)]
+         + [(n, False, False, True) for n in (3000, 10001)] + [(n, True, False, True) for n in (3000, 5377)])
+
+
+@pytest.mark.parametrize("n,angular,fp64,wall", CASES)
+def test_symmetric_product(orc, n, angular, fp64, wall):
+    pos, F, T = system(n, np.float64 if fp64 else np.float32, wall)
+    T = T if angular else None
+    out = []
+    for pinned in (False, True):
+        s = lm.lm_create(0.9, 1.0, angular, lm.LM_FP64 if fp64 else lm.LM_FP32C,
+                         periodicity=("open", "open", "single_wall" if wall else "open"))
+        lm.lm_set_positions(s, dev(pos))
+        if pinned:
+            c = lm.lm_get_pair_config(s)
+            lm.lm_set_pair_config(s, c["threads"], c["ilp"], c["splits"], c["packed"])
+        out.append([v for v in lm.lm_mdot(s, dev(F), dev(T)) if v is not None])
+        if not pinned:
+            again = [v for v in lm.lm_mdot(s, dev(F), dev(T)) if v is not None]
+            assert all(torch.equal(a, b) for a, b in zip(out[0], again))
+    rows = np.unique(np.concatenate([[0, 1, n // 2, n - 1], np.random.default_rng(1).integers(0, n, 200)]) % n)
+    ref = [v for v in orc.mdot(pos, F, T, 1.0, 0.9, angular, rows=rows, wall=wall) if v is not None]
+    # the product's bounds: 1e-12 (FP64), 1e-5 (FP32 compensated)
+    tol = 1e-12 if fp64 else 1e-5
+    for a, b, r in zip(*out, ref):
+        a, b = a.cpu().numpy(), b.cpu().numpy()
+        assert rel(a[rows], r) <= tol, (n, rel(a[rows], r))
+        assert rel(a, b) <= tol, (n, rel(a, b))
+
+
+@pytest.mark.parametrize("fp64,wall,n", [(False, False, 3100), (False, True, 3100), (True, False, 300)])
+def test_symmetric_product_in_the_square_root(fp64, wall, n):
+    """FP64 Krylov vectors enter the symmetric product and FP64 sums leave it."""
+    pos, _, _ = system(n, np.float64 if fp64 else np.float32, wall)
+    pos = pos[1:n - 1]   # without the coincident pair (M stays positive definite)
+    W = dev(np.random.default_rng(2).standard_normal(3 * len(pos)))
+    ys = []
+    for pinned in (False, True):
+        s = lm.lm_create(1.0, 1.0, False, lm.LM_FP64 if fp64 else lm.LM_FP32C,
+                         periodicity=("open", "open", "single_wall" if wall else "open"))
+        lm.lm_set_positions(s, dev(pos))
+        if pinned:
+            c = lm.lm_get_pair_config(s)
+            lm.lm_set_pair_config(s, c["threads"], c["ilp"], c["splits"], c["packed"])
+        ys.append(lm.lm_sqrt_mdot(s, W, tol=1e-4, max_iter=150)[0].double().cpu().numpy())
+    assert rel(ys[0], ys[1]) <= 20e-4   # each within 20 tol of the root
