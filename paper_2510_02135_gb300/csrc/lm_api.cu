@@ -163,10 +163,9 @@ struct lm_solver {
 
     // Lanczos state
     DBuf V, w, y, red, scal, zbuf, cbuf, Wbuf;
-    // symmetric adjoint: work-item table (for sym_key) and FP64 accumulators
-    DBuf sym_items, sym_acc;
-    std::array<int64_t, 4> sym_key{{-1, 0, 0, 0}};
-    int64_t sym_n_items = 0;
+    // plan of the symmetric adjoint, for (N, threads, ilp, splits, packed)
+    lmk::SymPlan adj_sym{};
+    std::array<int64_t, 5> adj_sym_key{{-1, 0, 0, 0, 0}};
     double* pinned = nullptr;  // host scalar read-back
     size_t pinned_doubles = 0;
 
@@ -516,26 +515,35 @@ bool valid_name(const char* p) {
 }  // namespace
 
 namespace {
-// Adjoint launch configuration (item sizes chosen at launch).  FP32 with
-// angular blocks: the symmetric packed form (packed = 4, ilp 4), 1.7x faster
-// than the one-sided scalar kernel at N = 65536; FP64: the symmetric scalar
-// form (packed = 3), 1.5x faster at N = 16384.  FP32 translation: the packed
-// one-sided kernel, packed = j-particles per overlap vote (the autotuner also
-// times the symmetric form).
-lm_pair_config default_adjoint_config(const lm_solver* s) {
-    if (s->fp64) return lm_pair_config{128, 1, 0, 3};
-    if (s->angular) return lm_pair_config{128, 4, 0, 4};
-    lm_pair_config c{128, lmk::adjoint_ilp(0, 0), 1, 1};
-    int occ = std::max(1, lmk::adjoint_ctas_per_sm(0, 0, c.threads, c.ilp, c.packed));
+// One-sided adjoint kernel with the model's splits.
+lm_pair_config one_sided_adjoint_config(const lm_solver* s) {
+    const bool tt = !s->fp64 && !s->angular;
+    lm_pair_config c{128, lmk::adjoint_ilp(s->fp64, s->angular), 1, tt ? 1 : 0};
+    int occ = std::max(1, lmk::adjoint_ctas_per_sm(s->fp64, s->angular, c.threads, c.ilp, c.packed));
     c.splits = auto_splits(s->N, c.threads, c.ilp, occ * s->sm_count);
     const int64_t nblk = (s->N + (int64_t)c.threads * c.ilp - 1) / ((int64_t)c.threads * c.ilp);
-    if (nblk * lmk::mdot_effective_splits(s->N, c.threads, c.splits) < (int64_t)occ * s->sm_count) {
+    if (tt && nblk * lmk::mdot_effective_splits(s->N, c.threads, c.splits) < (int64_t)occ * s->sm_count) {
         // too few CTAs to fill the GPU: the smaller i-blocks and splits of down to one j-tile
         c.ilp = 2;
         occ = std::max(1, lmk::adjoint_ctas_per_sm(0, 0, c.threads, c.ilp, c.packed));
         c.splits = auto_splits(s->N, c.threads, c.ilp, occ * s->sm_count, 1);
     }
     return c;
+}
+
+// Adjoint launch configuration (item sizes chosen at launch): the symmetric
+// kernels, except for small FP32 translation-only systems.  Time per call,
+// ilp 2 / 4 / one-sided: FP32 translation N = 2048 41 / - / 37 us, 3000 55 / 60
+// / 96, 4096 55 / 64 / 95, 8192 132 / 144 / 203, 16384 450 / 427 / 606, 65536
+// 6.61 / 6.27 / 8.43 ms; with angular blocks 1024 64 / 103 / 177 us, 4096 103 /
+// 109 / 174, 16384 1156 / 1061 / 1776, 65536 17.1 / 15.5 / 27.0 ms.  FP64 (ilp
+// 1): 1024 0.12 / 1.17 ms, 8001 4.97 / 8.48 ms; with angular blocks 4096 3.18 /
+// 5.91 ms.
+lm_pair_config default_adjoint_config(const lm_solver* s) {
+    if (s->fp64) return lm_pair_config{128, 1, 0, 3};
+    const int ilp = s->N <= 10000 ? 2 : 4;
+    if (s->angular) return lm_pair_config{128, ilp, 0, 4};
+    return s->N >= 3000 ? lm_pair_config{128, ilp, 0, 3} : one_sided_adjoint_config(s);
 }
 
 void ensure_adjoint_config(lm_solver* s) {
@@ -555,20 +563,6 @@ void ensure_adjoint_config(lm_solver* s) {
     s->adj_cfg_N = s->N;
 }
 
-// Tiles per work item of the symmetric adjoint when the configuration leaves
-// it open: about six items per resident CTA slot over the block-triangle of
-// (i-block, tile) units, and for the heavier angular and FP64 pairs at most
-// four tiles (4 against 8-19 was 2-3% faster at N = 65536 and 16384).
-int64_t sym_auto_chunk(const lm_solver* s, int threads, int ilp, int packed) {
-    const int64_t BI = (int64_t)threads * ilp;
-    const int64_t nblk = (s->N + BI - 1) / BI;
-    const int64_t T = (s->N + threads - 1) / threads;
-    const int occ = std::max(1, lmk::adjoint_ctas_per_sm(s->fp64, s->angular, threads, ilp, packed));
-    const double total = (double)nblk * (double)T - (double)ilp * (double)nblk * (double)(nblk - 1) / 2.0;
-    const int64_t chunk = std::max<int64_t>(1, (int64_t)std::ceil(total / (6.0 * occ * s->sm_count)));
-    return (s->fp64 || s->angular) ? std::min<int64_t>(chunk, 4) : chunk;
-}
-
 lm_status run_adjoint(lm_solver* s, const void* F, const void* T, const void* G, const void* H, void* dX, void* dF,
                       void* dT, const lm_pair_config& cfg) {
     lmk::AdjointArgs a;
@@ -586,33 +580,27 @@ lm_status run_adjoint(lm_solver* s, const void* F, const void* T, const void* G,
     a.splits = cfg.splits;
     a.partials = nullptr;
     if (a.uj >= 3) {
-        // symmetric form: items (i-block b, tiles [t0, t1)) over each block's
-        // tiles from its own range onward, at most `chunk` tiles each, longest first
-        const int64_t BI = (int64_t)cfg.threads * cfg.ilp;
-        const int64_t nblk = (s->N + BI - 1) / BI;
-        const int64_t T = (s->N + cfg.threads - 1) / cfg.threads;
-        const int64_t chunk = cfg.splits >= 1 ? cfg.splits : sym_auto_chunk(s, cfg.threads, cfg.ilp, a.uj);
-        const std::array<int64_t, 4> key{{s->N, cfg.threads, cfg.ilp, chunk}};
-        if (s->sym_key != key) {
-            std::vector<int4> items;
-            for (int64_t b = 0; b < nblk; ++b)
-                for (int64_t t0 = b * cfg.ilp; t0 < T; t0 += chunk)
-                    items.push_back(make_int4((int)b, (int)t0, (int)std::min(T, t0 + chunk), 0));
-            std::stable_sort(items.begin(), items.end(),
-                             [](const int4& x, const int4& y) { return (x.z - x.y) > (y.z - y.y); });
-            LM_CUDA(s->sym_items.ensure(items.size() * sizeof(int4)), "allocating adjoint work items");
-            LM_CUDA(cudaMemcpyAsync(s->sym_items.p, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice,
-                                    s->stream),
-                    "adjoint work items");
-            LM_CUDA(cudaStreamSynchronize(s->stream), "adjoint work items");
-            s->sym_key = key;
-            s->sym_n_items = (int64_t)items.size();
+        // symmetric form: its plan, and slots for both sides' sums
+        const std::array<int64_t, 5> key{{s->N, cfg.threads, cfg.ilp, cfg.splits, cfg.packed}};
+        if (s->adj_sym_key != key) {
+            lmk::adjoint_sym_tiling(s->fp64, cfg.threads, cfg.ilp, &s->adj_sym);
+            const int occ = std::max(1, lmk::adjoint_ctas_per_sm(s->fp64, s->angular, cfg.threads, cfg.ilp, a.uj));
+            // the configuration counts tiles of `threads` particles
+            const int64_t chunk =
+                cfg.splits >= 1 ? std::max<int64_t>(1, (int64_t)cfg.splits * cfg.threads / s->adj_sym.tile) : 0;
+            lmk::sym_layout(&s->adj_sym, s->N, lmk::adjoint_partial_components(s->angular),
+                            (int64_t)occ * s->sm_count, chunk);
+            s->adj_sym_key = key;
         }
-        LM_CUDA(s->sym_acc.ensure((size_t)lmk::adjoint_partial_components(s->angular) * s->N * sizeof(double)),
-                "allocating adjoint accumulators");
-        a.sym_items = s->sym_items.p;
-        a.n_sym_items = s->sym_n_items;
-        a.sym_acc = s->sym_acc.as<double>();
+        const size_t pb = (size_t)s->adj_sym.slots * lmk::adjoint_partial_components(s->angular) * (size_t)s->N *
+                          sizeof(double);
+        if (s->partials.ensure(pb) != cudaSuccess) {
+            // no room for the slots: the one-sided form, which needs fewer
+            cudaGetLastError();
+            return run_adjoint(s, F, T, G, H, dX, dF, dT, one_sided_adjoint_config(s));
+        }
+        a.sym = s->adj_sym;
+        a.partials = s->partials.as<double>();
         LM_CUDA(lmk::launch_adjoint(a, s->stream), "adjoint kernel");
         return LM_OK;
     }
@@ -1493,10 +1481,8 @@ lm_status autotune_impl(lm_solver* s, int reps, lm_pair_config* best) {
                     const int occ = lmk::adjoint_ctas_per_sm(0, 0, t, il, uj);
                     if (occ < 1) continue;
                     if (uj == 3) {
-                        // symmetric form: the item size (tiles) of the model, half and twice it
-                        const int64_t ch = sym_auto_chunk(s, t, il, 3);
-                        for (int64_t c : {ch, std::max<int64_t>(1, ch / 2), 2 * ch})
-                            acands.push_back(lm_pair_config{t, il, (int)std::min<int64_t>(c, 1 << 20), 3});
+                        // symmetric form: the item size of the model
+                        acands.push_back(lm_pair_config{t, il, 0, 3});
                         continue;
                     }
                     for (int sp : split_candidates(N, t, il, occ * s->sm_count))

@@ -159,6 +159,15 @@ struct MdotArgs {
     cudaEvent_t ev_end = nullptr;     // kernel when non-null (profiling)
 };
 
+// Plan of a symmetric kernel (sym_kernels.cu, adjoint_sym_kernels.cu): every
+// unordered pair once; slots * components * N doubles of partial sums.
+struct SymPlan {
+    int threads, ilp, tile;       // CTA size, i-particles per thread, particles per j-tile
+    int64_t tb, T;                // j-tiles per i-block, j-tiles
+    int64_t m, nsuper, chunk;     // i-blocks per superblock, superblocks, j-tiles per item
+    int64_t slots;
+};
+
 // Backward (adjoint) product.
 struct AdjointArgs {
     int fp64;
@@ -174,12 +183,8 @@ struct AdjointArgs {
     int uj = 1;                       // j-particles per overlap vote (packed form: 1 or 2); 3: symmetric
                                       // form (packed for FP32 translation, scalar otherwise); 4: symmetric
                                       // packed form with angular blocks (FP32)
-    double* partials;                 // splits * (3 + 3 or 6) * N doubles when splits > 1
-    // symmetric forms (uj >= 3): work items (int4: i-block, first tile, end tile, 0) and the
-    // FP64 accumulators acc[N][C], C = 6 or 9 with angular blocks (zeroed by the launcher)
-    const void* sym_items = nullptr;
-    int64_t n_sym_items = 0;
-    double* sym_acc = nullptr;
+    double* partials;                 // splits * (6 or 9) * N doubles when splits > 1; symmetric: slots of them
+    SymPlan sym{};                    // symmetric forms (uj >= 3)
 };
 
 // Launch-configuration tables (pair_kernels.cu / adjoint_kernels.cu).
@@ -197,17 +202,18 @@ cudaError_t launch_mdot(const MdotArgs& a, cudaStream_t s);
 bool wall_config_supported(int fp64, int threads, int ilp, int packed);
 int wall_ctas_per_sm(int fp64, int angular, int threads, int ilp, int packed);
 cudaError_t launch_wall_mdot(const MdotArgs& a, cudaStream_t s);
-// Symmetric form of the product (sym_kernels.cu): every unordered pair once.
-// slots * (3 or 6) * N doubles of partial sums.
-struct SymPlan {
-    int threads, ilp, tile;       // CTA size, i-particles per thread, particles per j-tile
-    int64_t tb, T;                // j-tiles per i-block, j-tiles
-    int64_t m, nsuper, chunk;     // i-blocks per superblock, superblocks, j-tiles per item
-    int64_t slots;
-};
 // The plan for a product that the symmetric form serves best, else false.
 bool sym_plan(int fp64, int angular, int wall, int64_t N, int sm_count, SymPlan* p);
+// Completes a plan whose threads, ilp and tile are set, for C components and
+// `resident` CTAs on the device: about eight items per resident CTA, or items
+// of `chunk` tiles when it is positive (more where the slots would exceed 128
+// or 256 MiB).
+void sym_layout(SymPlan* p, int64_t N, int C, int64_t resident, int64_t chunk);
 cudaError_t launch_sym_mdot(const MdotArgs& a, const SymPlan& p, int wall, cudaStream_t s);
+// Symmetric adjoint (AdjointArgs::uj 3 and 4): CTA tiling and launch.
+void adjoint_sym_tiling(int fp64, int threads, int ilp, SymPlan* p);
+int adjoint_sym_ctas_per_sm(int fp64, int angular, int threads, int ilp, int uj);
+cudaError_t launch_adjoint_sym(const AdjointArgs& a, cudaStream_t s);
 cudaError_t launch_adjoint(const AdjointArgs& a, cudaStream_t s);
 int adjoint_partial_components(int angular);
 int adjoint_ilp(int fp64, int angular);

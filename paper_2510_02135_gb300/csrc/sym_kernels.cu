@@ -29,86 +29,12 @@
 //     are bitwise reproducible.
 #include <cuda_runtime.h>
 
-#include <algorithm>
 #include <cstdint>
 
-#include "lm_internal.cuh"
-#include "pair_common.cuh"
+#include "sym_common.cuh"
 
 namespace lmk {
 namespace {
-
-struct SymGeom {
-    int64_t N, T;          // particles, j-tiles
-    int64_t m, chunk;      // i-blocks per superblock, j-tiles per item
-    int64_t tb;            // j-tiles per i-block
-    int64_t slots;         // FP64 slots of every (component, particle)
-    int64_t nsuper;        // superblocks
-};
-
-template <bool B>
-struct BoolTag {
-    static constexpr bool value = B;
-};
-
-struct SymItem {
-    int64_t S, c, t0, t1;  // superblock, chunk, first and end tile
-};
-
-__host__ __device__ inline int64_t sym_chunks(const SymGeom& g, int64_t S) {
-    return (g.T - S * g.m * g.tb + g.chunk - 1) / g.chunk;
-}
-
-// Item of this CTA; false past the end of its grid row.  Row y holds the
-// chunks of superblock y, then those of superblock nsuper - 1 - y: a long and
-// a short one, so that the rows are alike and hardly any CTA is empty (empty
-// CTAs would take a place on an SM while the items are dealt out).
-__device__ __forceinline__ bool sym_item(const SymGeom& g, SymItem* it) {
-    it->S = blockIdx.y;
-    it->c = blockIdx.x;
-    const int64_t n = sym_chunks(g, it->S);
-    if (it->c >= n) {
-        it->c -= n;
-        const int64_t S2 = g.nsuper - 1 - it->S;
-        if (S2 == it->S || it->c >= sym_chunks(g, S2)) return false;
-        it->S = S2;
-    }
-    it->t0 = it->S * g.m * g.tb + it->c * g.chunk;
-    const int64_t e = it->t0 + g.chunk;
-    it->t1 = e < g.T ? e : g.T;
-    return true;
-}
-
-// out = c8 f_i sum of particle i's slots: j-side slots of the earlier
-// superblocks (and of its own, unless it is in the superblock's first block),
-// then the i-side slots of its superblock's chunks.
-template <typename R>
-__global__ void sym_reduce_kernel(const double* __restrict__ partials, SymGeom g, int64_t block, int C, double c8,
-                                  const typename V4<R>::type* __restrict__ pos4, int wall, void* __restrict__ lin,
-                                  void* __restrict__ ang, int out_f64) {
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= (int64_t)C * g.N) return;
-    const int c = (int)(e / g.N);
-    const int64_t i = e - (int64_t)c * g.N;
-    const int64_t b = i / block, S = b / g.m;
-    const int64_t nj = S + ((b - S * g.m) > 0 ? 1 : 0);
-    const int64_t nc = sym_chunks(g, S);
-    const double* p = partials + (int64_t)c * g.N + i;
-    const int64_t stride = (int64_t)C * g.N;
-    double s0 = 0.0, s1 = 0.0;
-    int64_t k = 0;
-    for (; k + 2 <= nj; k += 2) { s0 += p[k * stride]; s1 += p[(k + 1) * stride]; }
-    if (k < nj) s0 += p[k * stride];
-    p += (S + 1) * stride;
-    for (k = 0; k + 2 <= nc; k += 2) { s0 += p[k * stride]; s1 += p[(k + 1) * stride]; }
-    if (k < nc) s0 += p[k * stride];
-    double s = s0 + s1;
-    if (wall) s *= (double)pos4[i].w;
-    void* out = (c < 3) ? lin : ang;
-    const int64_t idx = 3 * i + (c % 3);
-    if (out_f64) static_cast<double*>(out)[idx] = c8 * s;
-    else static_cast<float*>(out)[idx] = (float)(c8 * s);
-}
 
 // ---------------------------------------------------------------------------
 // Scalar form (FP64).  The FP64 pipe takes one warp instruction per 64 cycles
@@ -706,14 +632,6 @@ __global__ void __launch_bounds__(NT) sym_mdot_x2_kernel(const float4* __restric
     }
 }
 
-template <typename K>
-int occupancy_of(K kernel, int threads, size_t dyn) {
-    int n = 0;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, threads, dyn);
-    return e == cudaSuccess && n > 0 ? n : 1;
-}
-
 constexpr int kSymThreads = 128;
 constexpr int kSymWaves = 8;      // items per resident CTA: the largest leave at most an eighth of a wave idle
 constexpr int kTileF64 = 32;      // short tiles: small systems still give every SM an item
@@ -741,7 +659,7 @@ cudaError_t launch_sym_x2(const MdotArgs& a, const SymGeom& g, dim3 grid, cudaSt
 
 template <bool ANG, bool WALL, int NI>
 int occ_sym_x2() {
-    return occupancy_of(sym_mdot_x2_kernel<ANG, WALL, kSymThreads, NI, kTileF32>, kSymThreads,
+    return sym_occupancy(sym_mdot_x2_kernel<ANG, WALL, kSymThreads, NI, kTileF32>, kSymThreads,
                         sym_smem_bytes<ANG, kSymThreads, NI, kTileF32>());
 }
 
@@ -764,6 +682,26 @@ bool sym_selected(int fp64, int angular, int wall, int64_t N) {
     return N >= 3000 && (wall || !angular);
 }
 
+void sym_layout(SymPlan* p, int64_t N, int C, int64_t resident, int64_t chunk) {
+    const int64_t block = (int64_t)p->threads * p->ilp;
+    const int64_t nblk = (N + block - 1) / block;
+    p->tb = block / p->tile;
+    p->T = (N + p->tile - 1) / p->tile;
+    const int64_t units = nblk * p->T - p->tb * (nblk * (nblk - 1) / 2);
+    const int64_t most = std::max<int64_t>(128, ((int64_t)256 << 20) / ((int64_t)C * N * (int64_t)sizeof(double)));
+    for (p->m = 1;; p->m *= 2) {
+        p->nsuper = (nblk + p->m - 1) / p->m;
+        const int64_t want = chunk > 0 ? chunk : std::max<int64_t>(1, units / (kSymWaves * resident * p->m));
+        for (p->chunk = want;; p->chunk += want) {
+            p->slots = p->nsuper + 1;
+            for (int64_t S = 0; S < p->nsuper; ++S)
+                p->slots = std::max(p->slots, S + 1 + (p->T - S * p->m * p->tb + p->chunk - 1) / p->chunk);
+            if (p->slots <= most) return;
+            if (p->chunk > p->m * p->tb) break;
+        }
+    }
+}
+
 bool sym_plan(int fp64, int angular, int wall, int64_t N, int sm_count, SymPlan* p) {
     if (!sym_selected(fp64, angular, wall, N)) return false;
     p->threads = kSymThreads;
@@ -771,8 +709,8 @@ bool sym_plan(int fp64, int angular, int wall, int64_t N, int sm_count, SymPlan*
     int occ = 1;
     if (fp64) {
         p->ilp = 1;
-        occ = angular ? occupancy_of(sym_mdot_f64_kernel<true, kSymThreads, 1, kTileF64>, kSymThreads, 0)
-                      : occupancy_of(sym_mdot_f64_kernel<false, kSymThreads, 1, kTileF64>, kSymThreads, 0);
+        occ = angular ? sym_occupancy(sym_mdot_f64_kernel<true, kSymThreads, 1, kTileF64>, kSymThreads, 0)
+                      : sym_occupancy(sym_mdot_f64_kernel<false, kSymThreads, 1, kTileF64>, kSymThreads, 0);
     } else if (wall) {
         // i-particles per thread: more reuse of a j-value and fewer shuffles against more items.  Wall: 2
         // against 4, 8192: 153 / 166 us, 32768: 1.99 / 1.93 ms; free space 2 / 4 / 8, 8192: 73 / 76 / 75 us,
@@ -785,34 +723,14 @@ bool sym_plan(int fp64, int angular, int wall, int64_t N, int sm_count, SymPlan*
         occ = p->ilp == 2 ? occ_sym_x2<false, false, 2>()
                           : (p->ilp == 4 ? occ_sym_x2<false, false, 4>() : occ_sym_x2<false, false, 8>());
     }
-    const int64_t block = (int64_t)p->threads * p->ilp;
-    const int64_t C = angular ? 6 : 3;
-    const int64_t nblk = (N + block - 1) / block;
-    p->tb = block / p->tile;
-    p->T = (N + p->tile - 1) / p->tile;
-    const int64_t units = nblk * p->T - p->tb * (nblk * (nblk - 1) / 2);
-    const int64_t most = std::max<int64_t>(128, ((int64_t)256 << 20) / (C * N * (int64_t)sizeof(double)));
-    for (p->m = 1;; p->m *= 2) {
-        p->nsuper = (nblk + p->m - 1) / p->m;
-        const int64_t want = std::max<int64_t>(1, units / (kSymWaves * occ * sm_count * p->m));
-        for (p->chunk = want;; p->chunk += want) {
-            p->slots = p->nsuper + 1;
-            for (int64_t S = 0; S < p->nsuper; ++S)
-                p->slots = std::max(p->slots, S + 1 + (p->T - S * p->m * p->tb + p->chunk - 1) / p->chunk);
-            if (p->slots <= most) return true;
-            if (p->chunk > p->m * p->tb) break;
-        }
-    }
+    sym_layout(p, N, angular ? 6 : 3, (int64_t)std::max(1, occ) * sm_count, 0);
+    return true;
 }
 
 cudaError_t launch_sym_mdot(const MdotArgs& a, const SymPlan& p, int wall, cudaStream_t s) {
-    const SymGeom g{a.N, p.T, p.m, p.chunk, p.tb, p.slots, p.nsuper};
-    const int64_t rows = (p.nsuper + 1) / 2;
-    int64_t width = 0;
-    for (int64_t S = 0; S < rows; ++S)
-        width = std::max(width, sym_chunks(g, S) + (p.nsuper - 1 - S == S ? 0 : sym_chunks(g, p.nsuper - 1 - S)));
-    const dim3 grid((unsigned)width, (unsigned)rows);
-    if (rows > 65535 || a.partials == nullptr) return cudaErrorInvalidConfiguration;
+    const SymGeom g = sym_geom(a.N, p);
+    const dim3 grid = sym_grid(g);
+    if (grid.y > 65535 || a.partials == nullptr) return cudaErrorInvalidConfiguration;
     const double c8 = 1.0 / (8.0 * 3.14159265358979323846 * a.eta);
     if (a.ev_begin) cudaEventRecord(a.ev_begin, s);
     cudaError_t err;
@@ -830,16 +748,9 @@ cudaError_t launch_sym_mdot(const MdotArgs& a, const SymPlan& p, int wall, cudaS
     count_launches(1);
     if (err != cudaSuccess) return err;
     const int C = a.angular ? 6 : 3;
-    const unsigned blocks = (unsigned)(((int64_t)C * a.N + 127) / 128);
-    const int64_t block = (int64_t)p.threads * p.ilp;
-    if (a.fp64)
-        sym_reduce_kernel<double><<<blocks, 128, 0, s>>>(a.partials, g, block, C, c8,
-                                                         static_cast<const dvec4*>(a.pos4), wall, a.lin, a.ang, a.out_f64);
-    else
-        sym_reduce_kernel<float><<<blocks, 128, 0, s>>>(a.partials, g, block, C, c8,
-                                                        static_cast<const float4*>(a.pos4), wall, a.lin, a.ang, a.out_f64);
-    count_launches(1);
-    return cudaGetLastError();
+    const SymOut out{{a.lin, a.ang, nullptr}};
+    return a.fp64 ? launch_sym_reduce<double>(a.partials, p, g, C, c8, a.pos4, wall, out, a.out_f64, s)
+                  : launch_sym_reduce<float>(a.partials, p, g, C, c8, a.pos4, wall, out, a.out_f64, s);
 }
 
 }  // namespace lmk

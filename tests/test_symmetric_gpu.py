@@ -95,3 +95,32 @@ def test_symmetric_product_in_the_square_root(fp64, wall, n):
             lm.lm_set_pair_config(s, c["threads"], c["ilp"], c["splits"], c["packed"])
         ys.append(lm.lm_sqrt_mdot(s, W, tol=1e-4, max_iter=150)[0].double().cpu().numpy())
     assert rel(ys[0], ys[1]) <= 20e-4   # each within 20 tol of the root
+
+
+@pytest.mark.parametrize("n,angular,fp64", [(1, False, True), (2, True, True), (129, False, True), (300, True, True),
+                                            (129, True, False), (1000, True, False), (10241, True, False),
+                                            (3000, False, False), (10241, False, False), (66000, False, False)])
+def test_symmetric_adjoint(n, angular, fp64):
+    """The default adjoint against the one-sided kernel and bitwise against
+    itself; 66000 particles join i-blocks into superblocks."""
+    dt = np.float64 if fp64 else np.float32
+    pos, F, T = system(n, dt, False)
+    G, H = np.random.default_rng(3).standard_normal((2, n, 3)).astype(dt)
+    s = lm.lm_create(0.9, 1.0, angular, lm.LM_FP64 if fp64 else lm.LM_FP32C)
+    lm.lm_set_positions(s, dev(pos))
+    args = [dev(v) for v in ((F, T, G, H) if angular else (F, None, G, None))]
+    out = []
+    assert lm.lm_get_adjoint_config(s)["packed"] >= 3
+    for one_sided in (False, True):
+        if one_sided:
+            ilp = 1 if fp64 else (2 if angular else 4)
+            lm.lm_set_adjoint_config(s, 128, ilp, 0, 0 if fp64 or angular else 1)
+        out.append([v for v in lm.lm_mdot_backward(s, *args) if v is not None])
+        again = [v for v in lm.lm_mdot_backward(s, *args) if v is not None]
+        assert all(torch.equal(a, b) for a, b in zip(out[-1], again))
+    for a, b in zip(*out):   # the adjoint's bounds: 1e-12 (FP64), 1e-5 (FP32)
+        b = b.cpu().numpy()
+        if np.abs(b).max() > 0.0:
+            assert rel(a.cpu().numpy(), b) <= (1e-12 if fp64 else 1e-5), n
+        else:
+            assert not a.cpu().numpy().any()
