@@ -204,7 +204,7 @@ struct lm_solver {
         DBuf* all[] = {&pos4, &partials, &in_stage[0], &in_stage[1], &in_stage[2], &in_stage[3],
                        &out_stage[0], &out_stage[1], &out_stage[2], &flag, &tune_in, &tune_out,
                        &pos_raw, &rfd_pos4, &rfd_W, &rfd_P, &rfd_Q, &ab_u, &ab_d, &ab_y, &ab_x, &pc_p, &pc_q, &pc_t, &lzctr,
-                       &V, &w, &y, &red, &scal, &zbuf, &cbuf, &Wbuf, &sym_items, &sym_acc};
+                       &V, &w, &y, &red, &scal, &zbuf, &cbuf, &Wbuf};
         for (DBuf* b : all) b->release();
         if (pinned) cudaFreeHost(pinned);
         for (cudaEvent_t e : prof_ev) cudaEventDestroy(e);
