@@ -52,35 +52,53 @@ __device__ __forceinline__ bool sym_item(const SymGeom& g, SymItem* it) {
     return true;
 }
 
-// out = c8 f_i sum of particle i's slots: j-side slots of the earlier
-// superblocks (and of its own, unless it is in the superblock's first block),
-// then the i-side slots of its superblock's chunks.
 struct SymOut {
     void* o[3];            // components 0..2, 3..5, 6..8; null to skip
 };
 
+// out = c8 f_i sum of particle i's slots: j-side slots of the earlier
+// superblocks (and of its own, unless it is in the superblock's first block),
+// then the i-side slots of its superblock's chunks.  Bound by the latency of
+// its loads: the four warps of a CTA take a quarter of the slots of 32 values
+// each, eight loads in flight per thread (N = 4096, 33 slots: 14 us with two
+// loads in flight and one thread per value).
+constexpr int kReduceWarps = 4;
+
 template <typename R>
-__global__ void sym_reduce_kernel(const double* __restrict__ partials, SymGeom g, int64_t block, int C, double c8,
-                                  const typename V4<R>::type* __restrict__ pos4, int wall, SymOut out, int out_f64) {
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= (int64_t)C * g.N) return;
-    const int c = (int)(e / g.N);
+__global__ void __launch_bounds__(32 * kReduceWarps)
+    sym_reduce_kernel(const double* __restrict__ partials, SymGeom g, int64_t block, int C, double c8,
+                      const typename V4<R>::type* __restrict__ pos4, int wall, SymOut out, int out_f64) {
+    __shared__ double s_p[kReduceWarps][32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int64_t e = (int64_t)blockIdx.x * 32 + lane;
+    const bool in = e < (int64_t)C * g.N;
+    const int c = in ? (int)(e / g.N) : 0;
+    const int64_t i = in ? e - (int64_t)c * g.N : 0;
+    double s = 0.0;
+    if (in) {
+        const int64_t b = i / block, S = b / g.m;
+        const int nj = (int)(S + (b > S * g.m ? 1 : 0));
+        const int K = nj + (int)sym_chunks(g, S);
+        const int gap = (int)S + 1 - nj;   // slots skipped between the j-side and the i-side
+        const double* p = partials + (int64_t)c * g.N + i;
+        const int64_t stride = (int64_t)C * g.N;
+        const int k1 = K * (wid + 1) / kReduceWarps;
+        double t0 = 0.0, t1 = 0.0;
+        for (int k = K * wid / kReduceWarps; k < k1; k += 8) {
+            double v[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) v[q] = k + q < k1 ? p[(k + q < nj ? k + q : k + q + gap) * stride] : 0.0;
+#pragma unroll
+            for (int q = 0; q < 8; q += 2) { t0 += v[q]; t1 += v[q + 1]; }
+        }
+        s = t0 + t1;
+    }
+    s_p[wid][lane] = s;
+    __syncthreads();
+    if (wid != 0 || !in) return;
     void* dst = c < 3 ? out.o[0] : (c < 6 ? out.o[1] : out.o[2]);
     if (dst == nullptr) return;
-    const int64_t i = e - (int64_t)c * g.N;
-    const int64_t b = i / block, S = b / g.m;
-    const int64_t nj = S + ((b - S * g.m) > 0 ? 1 : 0);
-    const int64_t nc = sym_chunks(g, S);
-    const double* p = partials + (int64_t)c * g.N + i;
-    const int64_t stride = (int64_t)C * g.N;
-    double s0 = 0.0, s1 = 0.0;
-    int64_t k = 0;
-    for (; k + 2 <= nj; k += 2) { s0 += p[k * stride]; s1 += p[(k + 1) * stride]; }
-    if (k < nj) s0 += p[k * stride];
-    p += (S + 1) * stride;
-    for (k = 0; k + 2 <= nc; k += 2) { s0 += p[k * stride]; s1 += p[(k + 1) * stride]; }
-    if (k < nc) s0 += p[k * stride];
-    double s = s0 + s1;
+    s = (s + s_p[1][lane]) + (s_p[2][lane] + s_p[3][lane]);
     if (wall) s *= (double)pos4[i].w;
     const int64_t idx = 3 * i + (c % 3);
     if (out_f64) static_cast<double*>(dst)[idx] = c8 * s;
@@ -106,8 +124,8 @@ inline dim3 sym_grid(const SymGeom& g) {
 template <typename R>
 cudaError_t launch_sym_reduce(const double* partials, const SymPlan& p, const SymGeom& g, int C, double c8,
                               const void* pos4, int wall, SymOut out, int out_f64, cudaStream_t s) {
-    const unsigned blocks = (unsigned)(((int64_t)C * g.N + 127) / 128);
-    sym_reduce_kernel<R><<<blocks, 128, 0, s>>>(partials, g, (int64_t)p.threads * p.ilp, C, c8,
+    const unsigned blocks = (unsigned)(((int64_t)C * g.N + 31) / 32);
+    sym_reduce_kernel<R><<<blocks, 32 * kReduceWarps, 0, s>>>(partials, g, (int64_t)p.threads * p.ilp, C, c8,
                                                 static_cast<const typename V4<R>::type*>(pos4), wall, out, out_f64);
     count_launches(1);
     return cudaGetLastError();

@@ -635,51 +635,84 @@ __global__ void __launch_bounds__(NT) sym_mdot_x2_kernel(const float4* __restric
 constexpr int kSymThreads = 128;
 constexpr int kSymWaves = 8;      // items per resident CTA: the largest leave at most an eighth of a wave idle
 constexpr int kTileF64 = 32;      // short tiles: small systems still give every SM an item
-constexpr int kTileF32 = 128;
 
-template <bool ANG, int NI>
-cudaError_t launch_sym_f64(const MdotArgs& a, const SymGeom& g, dim3 grid, cudaStream_t s) {
-    sym_mdot_f64_kernel<ANG, kSymThreads, NI, kTileF64><<<grid, kSymThreads, 0, s>>>(
-        static_cast<const dvec4*>(a.pos4), a.F, ANG ? a.T : nullptr, a.in_f64, g, make_rpy_const<double>(a.a),
-        a.partials);
+// A form launches its kernel or, with occ, returns its resident CTAs per SM.
+template <bool ANG>
+cudaError_t f64_form(const MdotArgs* a, const SymGeom& g, dim3 grid, cudaStream_t s, int* occ) {
+    if (occ) {
+        *occ = sym_occupancy(sym_mdot_f64_kernel<ANG, kSymThreads, 1, kTileF64>, kSymThreads, 0);
+        return cudaSuccess;
+    }
+    sym_mdot_f64_kernel<ANG, kSymThreads, 1, kTileF64><<<grid, kSymThreads, 0, s>>>(
+        static_cast<const dvec4*>(a->pos4), a->F, ANG ? a->T : nullptr, a->in_f64, g, make_rpy_const<double>(a->a),
+        a->partials);
     return cudaGetLastError();
 }
 
-template <bool ANG, bool WALL, int NI>
-cudaError_t launch_sym_x2(const MdotArgs& a, const SymGeom& g, dim3 grid, cudaStream_t s) {
-    constexpr size_t dyn = sym_smem_bytes<ANG, kSymThreads, NI, kTileF32>();
+template <bool ANG, bool WALL, int NI, int TJ>
+cudaError_t x2_form(const MdotArgs* a, const SymGeom& g, dim3 grid, cudaStream_t s, int* occ) {
+    constexpr size_t dyn = sym_smem_bytes<ANG, kSymThreads, NI, TJ>();
+    if (occ) {
+        *occ = sym_occupancy(sym_mdot_x2_kernel<ANG, WALL, kSymThreads, NI, TJ>, kSymThreads, dyn);
+        return cudaSuccess;
+    }
     static std::atomic<unsigned long long> attr_devs{0};  // devices whose limit is raised
-    if (cudaError_t e = smem_attr_once(attr_devs, sym_mdot_x2_kernel<ANG, WALL, kSymThreads, NI, kTileF32>, dyn))
-        return e;
-    sym_mdot_x2_kernel<ANG, WALL, kSymThreads, NI, kTileF32><<<grid, kSymThreads, dyn, s>>>(
-        static_cast<const float4*>(a.pos4), a.F, ANG ? a.T : nullptr, a.in_f64, g, make_rpy_const<float>(a.a),
-        (float)(a.a * a.a), a.partials);
+    if (cudaError_t e = smem_attr_once(attr_devs, sym_mdot_x2_kernel<ANG, WALL, kSymThreads, NI, TJ>, dyn)) return e;
+    sym_mdot_x2_kernel<ANG, WALL, kSymThreads, NI, TJ><<<grid, kSymThreads, dyn, s>>>(
+        static_cast<const float4*>(a->pos4), a->F, ANG ? a->T : nullptr, a->in_f64, g, make_rpy_const<float>(a->a),
+        (float)(a->a * a->a), a->partials);
     return cudaGetLastError();
 }
 
-template <bool ANG, bool WALL, int NI>
-int occ_sym_x2() {
-    return sym_occupancy(sym_mdot_x2_kernel<ANG, WALL, kSymThreads, NI, kTileF32>, kSymThreads,
-                        sym_smem_bytes<ANG, kSymThreads, NI, kTileF32>());
+cudaError_t sym_form(int fp64, int angular, int wall, const SymPlan& p, const MdotArgs* a, const SymGeom& g, dim3 grid,
+                     cudaStream_t s, int* occ) {
+    if (fp64) return angular ? f64_form<true>(a, g, grid, s, occ) : f64_form<false>(a, g, grid, s, occ);
+#define LM_FORM(ANG, WALL, NI, TJ) \
+    if (angular == ANG && wall == WALL && p.ilp == NI && p.tile == TJ) return x2_form<ANG, WALL, NI, TJ>(a, g, grid, s, occ);
+    LM_FORM(false, false, 2, 32) LM_FORM(false, false, 2, 64) LM_FORM(false, false, 4, 128) LM_FORM(false, false, 8, 128)
+    LM_FORM(true, false, 2, 32) LM_FORM(true, false, 2, 64)
+    LM_FORM(false, true, 2, 32) LM_FORM(false, true, 2, 64) LM_FORM(false, true, 4, 128)
+    LM_FORM(true, true, 2, 32) LM_FORM(true, true, 2, 128)
+#undef LM_FORM
+    return cudaErrorInvalidConfiguration;
 }
 
 }  // namespace
 
-// Products that take the symmetric form (device time of one product on GB300,
-// symmetric / one-sided in its default configuration):
-//   FP64, free space: every N; N = 64: 53 / 178 us, 1024: 58 / 179 us, 8001:
-//     2.20 / 5.00 ms (all blocks: 104 / 315 us, 112 / 318 us, 4.88 / 8.17 ms);
-//   FP32 forces, free space: from N = 3000; 2048: 25.6 / 24.7 us, 4096: 30.9 /
-//     33.3, 8192: 68 / 84, 16384: 197 / 281, 65536: 2.57 / 3.26 ms;
-//   FP32 single wall: from N = 3000; 2048: 39.5 / 35.5 us, 4096: 56 / 73, 8192:
-//     148 / 214, 32768: 1.92 / 2.83 ms (all blocks: 66 / 50, 108 / 131, 324 /
-//     444 us, 4.73 / 5.97 ms).
-// FP32 with all blocks in free space stays one-sided: 46 against 41.5
-// operations do not pay for the j-side (N = 131072: 25.5 / 25.4 ms, 32768: 1.73
-// / 1.74 ms).  Neither does the FP64 wall, whose form is only scalar there.
-bool sym_selected(int fp64, int angular, int wall, int64_t N) {
-    if (fp64) return !wall;
-    return N >= 3000 && (wall || !angular);
+// Products that take the symmetric form.  FP64 with a wall does not (its
+// one-sided kernel has no packed form to share the wall part with), nor FP32
+// with all blocks in free space from N = 8000 on: 46 against 41.5 operations
+// do not pay for the j-side there (16384: 512 / 496 us, 131072: 25.5 / 25.4 ms).
+static bool sym_selected(int fp64, int angular, int wall, int64_t N) {
+    return wall ? !fp64 : (fp64 || !angular || N < 8000);
+}
+
+// i-particles per thread and particles per j-tile.  Small systems are bound by
+// the latency of one item, so short tiles and few i-particles make more and
+// shorter items; large ones by the FMA pipe, where more i-particles share a
+// j-value and its shuffles.  Device time of a product on GB300, us, symmetric
+// at (2, 32) / (2, 64) / (4, 128) / (8, 128) and one-sided with its default:
+//   forces, free space   N = 100   11 /  15 /  28 /    - |   22
+//                           1000   13 /  16 /  31 /    - |   24
+//                           4096   26 /  24 /  31 /    - |   33
+//                           8192   68 /  62 /  64 /    - |   84
+//                          16384  250 / 215 / 191 /  205 |  281
+//                          50021    - /   - /1570 / 1523 | 2164
+//   all blocks, free space  1000   15 /  22 |  27     4096  47 / 46 | 51     8192  148 / 136 | 138
+//   forces, wall            1000   16 /  23 /  60 |  36   4096  49 /  48 /  56 | 73
+//                          16384  518 / 518 / 498 | 779
+//   all blocks, wall, (2, 32) / (2, 128)   1000   23 / 66 | 51   4096   99 / 105 | 130
+//                          32768  4800 / 4724 | 5970
+//   FP64 (1 and 32, the FP64 pipe is full at one warp per SM quarter): forces 64: 53 | 178, 1000:
+//   54 | 179, 8001: 2193 | 4333; all blocks 64: 94 | 315, 1024: 109 | 318, 8001: 4859 | 8157
+static void sym_tiling(int fp64, int angular, int wall, int64_t N, int* ilp, int* tile) {
+    *ilp = fp64 ? 1 : 2;
+    *tile = 32;
+    if (fp64 || N < (angular && wall ? 5000 : 3500)) return;
+    *tile = angular && wall ? 128 : 64;
+    if (angular || N < 10000) return;
+    *tile = 128;
+    *ilp = wall || N < 40000 ? 4 : 8;
 }
 
 void sym_layout(SymPlan* p, int64_t N, int C, int64_t resident, int64_t chunk) {
@@ -705,24 +738,9 @@ void sym_layout(SymPlan* p, int64_t N, int C, int64_t resident, int64_t chunk) {
 bool sym_plan(int fp64, int angular, int wall, int64_t N, int sm_count, SymPlan* p) {
     if (!sym_selected(fp64, angular, wall, N)) return false;
     p->threads = kSymThreads;
-    p->tile = fp64 ? kTileF64 : kTileF32;
+    sym_tiling(fp64, angular, wall, N, &p->ilp, &p->tile);
     int occ = 1;
-    if (fp64) {
-        p->ilp = 1;
-        occ = angular ? sym_occupancy(sym_mdot_f64_kernel<true, kSymThreads, 1, kTileF64>, kSymThreads, 0)
-                      : sym_occupancy(sym_mdot_f64_kernel<false, kSymThreads, 1, kTileF64>, kSymThreads, 0);
-    } else if (wall) {
-        // i-particles per thread: more reuse of a j-value and fewer shuffles against more items.  Wall: 2
-        // against 4, 8192: 153 / 166 us, 32768: 1.99 / 1.93 ms; free space 2 / 4 / 8, 8192: 73 / 76 / 75 us,
-        // 16384: 217 / 203 / 214 us, 50021: 1.74 / 1.59 / 1.54 ms; wall with all blocks 2 at every size
-        p->ilp = angular || N <= 10000 ? 2 : 4;
-        occ = angular ? occ_sym_x2<true, true, 2>()
-                      : (p->ilp == 2 ? occ_sym_x2<false, true, 2>() : occ_sym_x2<false, true, 4>());
-    } else {
-        p->ilp = N <= 10000 ? 2 : (N <= 40000 ? 4 : 8);
-        occ = p->ilp == 2 ? occ_sym_x2<false, false, 2>()
-                          : (p->ilp == 4 ? occ_sym_x2<false, false, 4>() : occ_sym_x2<false, false, 8>());
-    }
+    if (sym_form(fp64, angular, wall, *p, nullptr, SymGeom{}, dim3(), nullptr, &occ) != cudaSuccess) return false;
     sym_layout(p, N, angular ? 6 : 3, (int64_t)std::max(1, occ) * sm_count, 0);
     return true;
 }
@@ -733,17 +751,7 @@ cudaError_t launch_sym_mdot(const MdotArgs& a, const SymPlan& p, int wall, cudaS
     if (grid.y > 65535 || a.partials == nullptr) return cudaErrorInvalidConfiguration;
     const double c8 = 1.0 / (8.0 * 3.14159265358979323846 * a.eta);
     if (a.ev_begin) cudaEventRecord(a.ev_begin, s);
-    cudaError_t err;
-    if (a.fp64)
-        err = a.angular ? launch_sym_f64<true, 1>(a, g, grid, s) : launch_sym_f64<false, 1>(a, g, grid, s);
-    else if (wall)
-        err = a.angular ? launch_sym_x2<true, true, 2>(a, g, grid, s)
-                        : (p.ilp == 2 ? launch_sym_x2<false, true, 2>(a, g, grid, s)
-                                      : launch_sym_x2<false, true, 4>(a, g, grid, s));
-    else
-        err = p.ilp == 2 ? launch_sym_x2<false, false, 2>(a, g, grid, s)
-                         : (p.ilp == 4 ? launch_sym_x2<false, false, 4>(a, g, grid, s)
-                                       : launch_sym_x2<false, false, 8>(a, g, grid, s));
+    const cudaError_t err = sym_form(a.fp64, a.angular, wall, p, &a, g, grid, s, nullptr);
     if (a.ev_end) cudaEventRecord(a.ev_end, s);
     count_launches(1);
     if (err != cudaSuccess) return err;
