@@ -22,6 +22,7 @@
 #include "lm_internal.cuh"
 #include "lm_runtime.cuh"
 #include "tridiag.cuh"
+#include "tridiag_quad.h"
 
 namespace {
 
@@ -97,8 +98,15 @@ bool is_device_ptr(const void* p) {
 struct LanczosHost {
     std::vector<double> alpha, beta, z, zprev, d, e, rc, rs;
     std::vector<int> rk;
+    lmk::SqrtQuadrature quad;
+    // z = normW sqrt(T) e1: quadrature where T is safely definite, else QR with negative Ritz values clamped
     int solve(int m, double normW, int* clamped) {
         z.assign(m, 0.0);
+        if (quad.solve(m, alpha.data(), beta.data(), z.data())) {
+            for (double& v : z) v *= normW;
+            *clamped = 0;
+            return 0;
+        }
         d.resize(m);
         e.resize(m);
         size_t max_rot = (size_t)4 * m * m + 64;
