@@ -10,6 +10,7 @@
 #include <cstdint>
 
 #include "lm_internal.cuh"
+#include "pdl.cuh"
 #include "philox.cuh"
 
 namespace lmk {
@@ -23,34 +24,6 @@ inline int blocks_for(int64_t n, int per_thread = 4) {
     if (b < 1) b = 1;
     if (b > kMaxBlocks) b = kMaxBlocks;
     return (int)b;
-}
-
-// Programmatic dependent launch: the per-iteration vector kernels are
-// launched with cudaLaunchAttributeProgrammaticStreamSerialization, so that
-// each can be scheduled while its predecessor in the stream drains.  Every
-// such kernel first waits for its predecessors to complete (griddepcontrol.
-// wait: their memory operations are then visible), so the order of all
-// memory accesses is that of plain stream order; only the launch latency
-// overlaps.  It then allows its own dependent to be scheduled.  In a launch
-// without the attribute both instructions return at once.
-__device__ __forceinline__ void pdl_enter() {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
-template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t s, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -359,6 +332,249 @@ __global__ void sub_vc_norm_kernel(const double* __restrict__ V, int m, const do
     if (threadIdx.x == 0) { out[0] = sqrt(t); out[1] = t; *ctr = 0u; }
 }
 
+// ---------------------------------------------------------------------------
+// Everything of a Lanczos iteration after its product, in one cooperative
+// launch: alpha, the three-term update, the Gram-Schmidt pass (and the second
+// one where the DGKS test asks for it), beta and v_{k+1} = w / beta.
+//
+// For vectors of up to 152 x 512 elements the launches of the separate kernels
+// cost more than their work (time per iteration with its product, separate /
+// here: N = 300 57 / 36 us, 4096 70 / 49, 16000 238 / 222, FP64 N = 1024 95 /
+// 75).  What bounds it is latency: three meetings of about 1 us, and chains of
+// FP64 adds of 64 cycles each.  Here CTA b owns the elements
+// [b E, (b + 1) E) and keeps its part of w in shared memory; the grid meets
+// three times (alpha; norm and dots; norm), and after each meeting every CTA
+// adds the CTAs' partial sums itself, all in the same order, so that no
+// further meeting distributes the totals and every CTA takes the same branch.
+// Dots: a warp takes eight rows at a time (eight FP64 chains, one transposing
+// butterfly); the subtraction splits the rows over 256 / E threads per element.
+// The CTAs wait for one another, so the launch is cooperative (all resident)
+// and every wait has a limit, after which the kernel sets the scalars' error
+// word and returns (the host then reports LM_ERR_TIMEOUT).
+// ---------------------------------------------------------------------------
+constexpr int kStepThreads = 256;
+constexpr long long kStepSpinCycles = 4000000000ll;   // about 2 s
+
+__device__ __forceinline__ bool step_meet(unsigned* ctr, unsigned* target) {
+    __shared__ int ok;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        *target += gridDim.x;
+        atomicAdd(ctr, 1u);
+        const long long t0 = clock64();
+        bool in = true;
+        while ((int)(*(volatile unsigned*)ctr - *target) < 0) {
+            if (clock64() - t0 > kStepSpinCycles) { in = false; break; }
+        }
+        __threadfence();
+        ok = in;
+    }
+    __syncthreads();
+    return ok != 0;
+}
+
+// Eight per-lane sums added over the warp: lane l returns the total of value l >> 2.
+__device__ __forceinline__ double warp_sum8(double (&v)[8], int lane) {
+#pragma unroll
+    for (int h = 4, o = 16; h >= 1; h >>= 1, o >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int r = 0; r < h; ++r) {
+            const double keep = up ? v[r + h] : v[r], send = up ? v[r] : v[r + h];
+            v[r] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+    }
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+    return v[0];
+}
+
+// Sum of this CTA's per-thread values to part[blockIdx.x] (thread 0 writes).
+__device__ __forceinline__ void step_put(double v, double* part) {
+    v = block_sum(v);
+    if (threadIdx.x == 0) part[blockIdx.x] = v;
+}
+
+// Sum of the CTAs' values, the same in every CTA; valid in every thread.
+__device__ __forceinline__ double step_total(const double* part) {
+    __shared__ double tot;
+    double v = 0.0;
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += kStepThreads) v += __ldcg(part + b);
+    v = block_sum(v);
+    if (threadIdx.x == 0) tot = v;
+    __syncthreads();
+    v = tot;
+    __syncthreads();
+    return v;
+}
+
+// One Gram-Schmidt pass over the rows [0, m): w -= V (V^T w) on this CTA's
+// elements.  |w|^2 before the pass is added up as one more row of the dots
+// (h0sq), |w|^2 after it by a third meeting (h1sq).  Returns false when a wait
+// ran out.
+template <int E>
+__device__ __forceinline__ bool step_gram_schmidt(const double* __restrict__ V, int m, int64_t n, int64_t e0, double* s_w,
+                                                  double* s_c, double* rows, double* norm1, double* h0sq, double* h1sq,
+                                                  unsigned* ctr, unsigned* target) {
+    constexpr int kPer = E / 32;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int G = gridDim.x;
+    double we[kPer];
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) we[q] = s_w[q * 32 + lane];
+    for (int j0 = wid * 8; j0 <= m; j0 += kStepThreads / 4) {
+        // rows and elements past the end load the last ones (finite, then not used, or times w = 0), so that
+        // no branch keeps the loads of two element columns from being in flight together
+        const double* __restrict__ row[8];
+        double acc[8];
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            row[r] = V + (int64_t)(j0 + r < m ? j0 + r : m - 1) * n;
+            acc[r] = 0.0;
+        }
+#pragma unroll
+        for (int q = 0; q < kPer; q += 2) {
+            double x[2][8];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int64_t e = e0 + (q + h) * 32 + lane;
+                const int64_t ec = e < n ? e : n - 1;
+#pragma unroll
+                for (int r = 0; r < 8; ++r) x[h][r] = row[r][ec];
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+#pragma unroll
+                for (int r = 0; r < 8; ++r) acc[r] = fma(j0 + r < m ? x[h][r] : we[q + h], we[q + h], acc[r]);
+            }
+        }
+        const double t = warp_sum8(acc, lane);
+        if ((lane & 3) == 0 && j0 + (lane >> 2) <= m) rows[(int64_t)(j0 + (lane >> 2)) * G + blockIdx.x] = t;
+    }
+    if (!step_meet(ctr, target)) return false;
+    for (int j0 = wid * 8; j0 <= m; j0 += kStepThreads / 4) {
+        double acc[8];
+#pragma unroll
+        for (int r = 0; r < 8; ++r) acc[r] = 0.0;
+#pragma unroll
+        for (int q = 0; q < 5; ++q) {   // at most 152 CTAs
+            const int b = q * 32 + lane;
+            if (q * 32 >= G) break;
+            double x[8];
+#pragma unroll
+            for (int r = 0; r < 8; ++r)
+                x[r] = __ldcg(rows + (int64_t)(j0 + r <= m ? j0 + r : m) * G + (b < G ? b : G - 1));
+#pragma unroll
+            for (int r = 0; r < 8; ++r) acc[r] += b < G ? x[r] : 0.0;
+        }
+        const double t = warp_sum8(acc, lane);
+        if ((lane & 3) == 0 && j0 + (lane >> 2) <= m) s_c[j0 + (lane >> 2)] = t;
+    }
+    __syncthreads();
+    *h0sq = s_c[m];
+    // subtraction: kGroups threads share an element's rows (or a thread takes E / 256 elements)
+    constexpr int kGroups = E < kStepThreads ? kStepThreads / E : 1;
+    constexpr int kElems = E > kStepThreads ? E / kStepThreads : 1;
+    __shared__ double s_p[kGroups > 1 ? kStepThreads : 1];
+    double v = 0.0;
+#pragma unroll
+    for (int q = 0; q < kElems; ++q) {
+        const int el = (tid % E) + q * kStepThreads, grp = tid / E;
+        const int64_t e = e0 + el;
+        double a0 = 0.0, a1 = 0.0;
+        if (e < n) {
+            int j = grp;
+            for (; j + kGroups < m; j += 2 * kGroups) {
+                a0 = fma(s_c[j], V[(int64_t)j * n + e], a0);
+                a1 = fma(s_c[j + kGroups], V[(int64_t)(j + kGroups) * n + e], a1);
+            }
+            if (j < m) a0 = fma(s_c[j], V[(int64_t)j * n + e], a0);
+        }
+        double t = a0 + a1;
+        if constexpr (kGroups > 1) {
+            s_p[tid] = t;
+            __syncthreads();
+#pragma unroll
+            for (int x = 1; x < kGroups; ++x) t += s_p[(tid + x * E) % kStepThreads];
+        }
+        if (grp == 0) {   // other groups hold the same elements
+            t = s_w[el] - t;
+            s_w[el] = t;
+            v = fma(t, t, v);
+        }
+    }
+    step_put(v, norm1);
+    if (!step_meet(ctr, target)) return false;
+    *h1sq = step_total(norm1);
+    return true;
+}
+
+// host_sc: the iteration's scalars [alpha, beta, beta^2, expired wait, -, h0^2,
+// -, h1^2] in page-locked host memory (a copy between two iterations would
+// hold up the second one's product); sc[1]: beta for the next iteration;
+// beta_prev: beta of the iteration before (null at k = 0); part: scratch of
+// (5 + 2 m) gridDim.x doubles, m = k + 1; *ctr is a multiple of gridDim.x.
+template <int E>
+__global__ void __launch_bounds__(kStepThreads) lanczos_step_kernel(double* __restrict__ V, int k,
+                                                                    const double* __restrict__ w, int64_t n,
+                                                                    double* sc, const double* beta_prev,
+                                                                    double* part, unsigned* ctr, int always_twice,
+                                                                    double* host_sc) {
+    __shared__ double s_w[E];
+    extern __shared__ double s_c[];   // k + 1 coefficients, |w|^2
+    const int tid = threadIdx.x, G = gridDim.x, m = k + 1;
+    const int64_t e0 = (int64_t)blockIdx.x * E;
+    const double* vk = V + (int64_t)k * n;
+    unsigned target = 0;
+    if (tid == 0) target = *(volatile unsigned*)ctr / G * G;
+    double dot = 0.0;
+    for (int q = tid; q < E; q += kStepThreads) {
+        const int64_t e = e0 + q;
+        const double x = e < n ? w[e] : 0.0;
+        s_w[q] = x;
+        if (e < n) dot = fma(x, vk[e], dot);
+    }
+    bool ok = true;
+    double alpha = 0.0, h0sq = 0.0, h1sq = 0.0, bsq = 0.0;
+    step_put(dot, part);
+    ok = step_meet(ctr, &target);
+    if (ok) {
+        alpha = step_total(part);
+        const double b = beta_prev != nullptr ? beta_prev[0] : 0.0;
+        for (int q = tid; q < E; q += kStepThreads) {
+            const int64_t e = e0 + q;
+            if (e < n) {
+                double x = s_w[q] - alpha * vk[e];
+                if (beta_prev != nullptr) x -= b * vk[e - n];
+                s_w[q] = x;
+            }
+        }
+        __syncthreads();
+        double* rows = part + 3 * (int64_t)G;
+        ok = step_gram_schmidt<E>(V, m, n, e0, s_w, s_c, rows, part + G, &h0sq, &h1sq, ctr, &target);
+        bsq = h1sq;
+        double again = 0.0;
+        if (ok && (always_twice || h1sq < 0.5 * h0sq))
+            ok = step_gram_schmidt<E>(V, m, n, e0, s_w, s_c, rows + (int64_t)(m + 1) * G, part + 2 * G, &again, &bsq, ctr,
+                                      &target);
+    }
+    if (!ok) {
+        if (tid == 0) host_sc[3] = 1.0;
+        return;
+    }
+    const double inv = rsqrt(bsq), beta = bsq == 0.0 ? 0.0 : bsq * inv;
+    for (int q = tid; q < E; q += kStepThreads) {
+        const int64_t e = e0 + q;
+        if (e < n) V[(int64_t)m * n + e] = s_w[q] * inv;
+    }
+    if (blockIdx.x == 0 && tid == 0) {
+        sc[1] = beta;
+        host_sc[0] = alpha; host_sc[1] = beta; host_sc[2] = bsq;
+        host_sc[5] = h0sq; host_sc[7] = h1sq;
+    }
+}
+
 inline int md_blocks(int64_t n) { return (int)((n + kMdChunk - 1) / kMdChunk); }
 
 }  // namespace
@@ -381,13 +597,13 @@ cudaError_t lz_norm(const double* x, int64_t n, double* red, double* out, cudaSt
 cudaError_t lz_dot1(const double* x, const double* y, int64_t n, double* red, unsigned* ctr, double* out,
                     int mode, cudaStream_t s) {
     count_launches(1);
-    return launch_pdl(dot_fused, dim3(blocks_for(n)), dim3(kThreads), s, x, y, n, red, ctr, out, mode);
+    return launch_pdl(dot_fused, dim3(blocks_for(n)), dim3(kThreads), 0, s, x, y, n, red, ctr, out, mode);
 }
 
 cudaError_t lz_axpy2_norm(double* w, const double* vk, const double* alpha, const double* vkm1, const double* beta,
                           int64_t n, double* red, unsigned* ctr, double* out, cudaStream_t s) {
     count_launches(1);
-    return launch_pdl(axpy2_norm_kernel, dim3(blocks_for(n)), dim3(kThreads), s, w, vk, alpha, vkm1, beta, n, red,
+    return launch_pdl(axpy2_norm_kernel, dim3(blocks_for(n)), dim3(kThreads), 0, s, w, vk, alpha, vkm1, beta, n, red,
                       ctr, out);
 }
 
@@ -397,20 +613,47 @@ cudaError_t lz_multidot1(const double* V, int m, const double* w, int64_t n, dou
     const int nb = md_blocks(n), ng = (m + kMdRows - 1) / kMdRows;
     if (nb < 1 || ng > 65535) return cudaErrorInvalidConfiguration;
     count_launches(1);
-    return launch_pdl(multidot_rows, dim3((unsigned)nb, (unsigned)ng), dim3(kMdThreads), s, V, m, w, n, red, ctr + 1, c,
+    return launch_pdl(multidot_rows, dim3((unsigned)nb, (unsigned)ng), dim3(kMdThreads), 0, s, V, m, w, n, red, ctr + 1, c,
                       cond);
 }
 
 cudaError_t lz_sub_vc_norm(const double* V, int m, const double* c, double* w, int64_t n, double* red,
                            unsigned* ctr, double* out, cudaStream_t s, const double* cond) {
     count_launches(1);
-    return launch_pdl(sub_vc_norm_kernel, dim3(blocks_for(n, 1)), dim3(kThreads), s, V, m, c, w, n, cond, red, ctr,
+    return launch_pdl(sub_vc_norm_kernel, dim3(blocks_for(n, 1)), dim3(kThreads), 0, s, V, m, c, w, n, cond, red, ctr,
                       out);
+}
+
+// Elements per CTA of the one-launch iteration: at most one CTA per SM (152).
+static int step_elems(int64_t n) {
+    for (int E = 64; E <= 512; E *= 2)
+        if (n <= (int64_t)152 * E) return E;
+    return 0;
+}
+
+size_t lz_step_doubles(int64_t n, int m_max) {
+    const int E = step_elems(n);
+    if (E == 0 || m_max > 4096) return 0;
+    return (size_t)((n + E - 1) / E) * (5 + 2 * (size_t)m_max);
+}
+
+cudaError_t lz_step(double* V, int k, const double* w, int64_t n, double* sc, const double* beta_prev, double* part,
+                    unsigned* ctr, int always_twice, double* host_sc, cudaStream_t s) {
+    const int E = step_elems(n);
+    const dim3 grid((unsigned)((n + E - 1) / E));
+    const size_t dyn = (size_t)(k + 2) * sizeof(double);
+    void* args[] = {&V, &k, &w, &n, &sc, &beta_prev, &part, &ctr, &always_twice, &host_sc};
+    const void* f = E == 64    ? (const void*)lanczos_step_kernel<64>
+                    : E == 128 ? (const void*)lanczos_step_kernel<128>
+                    : E == 256 ? (const void*)lanczos_step_kernel<256>
+                               : (const void*)lanczos_step_kernel<512>;
+    count_launches(1);
+    return cudaLaunchCooperativeKernel(f, grid, dim3(kStepThreads), args, dyn, s);
 }
 
 cudaError_t lz_scale(const double* x, const double* nrm, double* y, int64_t n, cudaStream_t s) {
     count_launches(1);
-    return launch_pdl(scale_kernel, dim3(blocks_for(n)), dim3(kThreads), s, x, nrm, y, n);
+    return launch_pdl(scale_kernel, dim3(blocks_for(n)), dim3(kThreads), 0, s, x, nrm, y, n);
 }
 
 cudaError_t lz_combine(const double* V, int m, const double* z, double* y, int64_t n, cudaStream_t s) {

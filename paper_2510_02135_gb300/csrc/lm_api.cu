@@ -167,6 +167,8 @@ struct lm_solver {
     DBuf pc_p, pc_q, pc_t;
     // device counter of the single-launch reductions (zero between launches)
     DBuf lzctr;
+    DBuf lzmeet;            // meeting counter of the one-launch iteration
+    bool lz_one = false;    // this call's iterations take one launch after the product
     uint64_t rfd_calls = 0;
 
     // Lanczos state
@@ -211,7 +213,7 @@ struct lm_solver {
     ~lm_solver() {
         DBuf* all[] = {&pos4, &partials, &in_stage[0], &in_stage[1], &in_stage[2], &in_stage[3],
                        &out_stage[0], &out_stage[1], &out_stage[2], &flag, &tune_in, &tune_out,
-                       &pos_raw, &rfd_pos4, &rfd_W, &rfd_P, &rfd_Q, &ab_u, &ab_d, &ab_y, &ab_x, &pc_p, &pc_q, &pc_t, &lzctr,
+                       &pos_raw, &rfd_pos4, &rfd_W, &rfd_P, &rfd_Q, &ab_u, &ab_d, &ab_y, &ab_x, &pc_p, &pc_q, &pc_t, &lzctr, &lzmeet,
                        &V, &w, &y, &red, &scal, &zbuf, &cbuf, &Wbuf};
         for (DBuf* b : all) b->release();
         if (pinned) cudaFreeHost(pinned);
@@ -1031,7 +1033,7 @@ lm_status lm_ab_step(lm_solver* s, const void* forces, const void* torques, cons
 namespace {
 
 // Device scalars per iteration k at scal + kScal * k:
-//   [alpha, beta, beta^2, -, h0, h0^2, h1, h1^2]
+//   [alpha, beta, beta^2, expired wait, h0, h0^2, h1, h1^2]
 constexpr int kScal = 8;
 
 lm_status enqueue_lanczos_iteration(lm_solver* s, int k, int64_t n, double* V, double* w, double* scal, double* red,
@@ -1039,7 +1041,7 @@ lm_status enqueue_lanczos_iteration(lm_solver* s, int k, int64_t n, double* V, d
     const int64_t N = s->N;
     double* vk = V + (int64_t)k * n;
     double* sk = scal + kScal * k;
-    if (k > 0) LM_CUDA(lmk::lz_scale(w, sk - kScal + 1, vk, n, s->stream), "next basis vector");
+    if (k > 0 && !s->lz_one) LM_CUDA(lmk::lz_scale(w, sk - kScal + 1, vk, n, s->stream), "next basis vector");
     if (s->precond) {
         // w = P M P v_k, P = diag(M)^{-1/2}
         double* t = s->pc_t.as<double>();
@@ -1065,21 +1067,28 @@ lm_status enqueue_lanczos_iteration(lm_solver* s, int k, int64_t n, double* V, d
         vend = s->vprof_ev[2 * s->vprof_used + 1];
         s->vprof_used += 1;
     }
-    LM_CUDA(lmk::lz_dot1(vk, w, n, red, ctr, sk, 0, s->stream), "alpha");
-    // three-term update and |w| before the Gram-Schmidt pass
-    LM_CUDA(lmk::lz_axpy2_norm(w, vk, sk, k > 0 ? vk - n : nullptr, k > 0 ? sk - kScal + 1 : nullptr, n, red, ctr,
-                               sk + 4, s->stream),
-            "three-term update");
-    // full reorthogonalisation: one Gram-Schmidt pass (|w| after it), a second
-    // one only after cancellation (DGKS); beta = |w| at the end
-    LM_CUDA(lmk::lz_multidot1(V, k + 1, w, n, red, ctr, cb, s->stream), "reorthogonalisation");
-    LM_CUDA(lmk::lz_sub_vc_norm(V, k + 1, cb, w, n, red, ctr, sk + 6, s->stream), "reorthogonalisation");
-    const double* cond = s->reorth ? nullptr : sk + 4;   // nullptr: the second pass always runs
-    LM_CUDA(lmk::lz_multidot1(V, k + 1, w, n, red, ctr, cb, s->stream, cond), "reorthogonalisation");
-    LM_CUDA(lmk::lz_sub_vc_norm(V, k + 1, cb, w, n, red, ctr, sk + 1, s->stream, cond), "beta");
+    if (s->lz_one) {
+        LM_CUDA(lmk::lz_step(V, k, w, n, sk, k > 0 ? sk - kScal + 1 : nullptr, red,
+                             s->lzmeet.as<unsigned>(), s->reorth, s->pinned + kScal * k, s->stream),
+                "Lanczos iteration");
+    } else {
+        LM_CUDA(lmk::lz_dot1(vk, w, n, red, ctr, sk, 0, s->stream), "alpha");
+        // three-term update and |w| before the Gram-Schmidt pass
+        LM_CUDA(lmk::lz_axpy2_norm(w, vk, sk, k > 0 ? vk - n : nullptr, k > 0 ? sk - kScal + 1 : nullptr, n, red, ctr,
+                                   sk + 4, s->stream),
+                "three-term update");
+        // full reorthogonalisation: one Gram-Schmidt pass (|w| after it), a second
+        // one only after cancellation (DGKS); beta = |w| at the end
+        LM_CUDA(lmk::lz_multidot1(V, k + 1, w, n, red, ctr, cb, s->stream), "reorthogonalisation");
+        LM_CUDA(lmk::lz_sub_vc_norm(V, k + 1, cb, w, n, red, ctr, sk + 6, s->stream), "reorthogonalisation");
+        const double* cond = s->reorth ? nullptr : sk + 4;   // nullptr: the second pass always runs
+        LM_CUDA(lmk::lz_multidot1(V, k + 1, w, n, red, ctr, cb, s->stream, cond), "reorthogonalisation");
+        LM_CUDA(lmk::lz_sub_vc_norm(V, k + 1, cb, w, n, red, ctr, sk + 1, s->stream, cond), "beta");
+    }
     if (vend) LM_CUDA(cudaEventRecord(vend, s->stream), "profiling event");
-    LM_CUDA(cudaMemcpyAsync(s->pinned + kScal * k, sk, kScal * sizeof(double), cudaMemcpyDeviceToHost, s->stream),
-            "read alpha, beta");
+    if (!s->lz_one)
+        LM_CUDA(cudaMemcpyAsync(s->pinned + kScal * k, sk, kScal * sizeof(double), cudaMemcpyDeviceToHost, s->stream),
+                "read alpha, beta");
     LM_CUDA(cudaEventRecord(ev, s->stream), "iteration event");
     return LM_OK;
 }
@@ -1100,7 +1109,7 @@ double lanczos_vector_bytes(int k, int64_t n, bool second_pass) {
 void settle_vector_profile(lm_solver* s, int64_t n) {
     for (const auto& pk : s->vprof_pending) {
         const double* sc = s->pinned + kScal * pk.second;
-        const bool second = s->reorth != 0 || sc[6] < sc[4] * 0.70710678118654752440;   // the kernels' DGKS test
+        const bool second = s->reorth != 0 || sc[7] < 0.5 * sc[5];   // the DGKS test on the squares
         if (pk.first < s->vprof_bytes.size()) s->vprof_bytes[pk.first] = lanczos_vector_bytes(pk.second, n, second);
     }
     s->vprof_pending.clear();
@@ -1135,7 +1144,10 @@ static lm_status sqrt_mdot_body(lm_solver* s, const double* W, uint64_t seed, do
     LM_CUDA(s->V.ensure((size_t)(m_max + 1) * n * sizeof(double)), "allocating Krylov basis");
     LM_CUDA(s->w.ensure((size_t)n * sizeof(double)), "allocating Lanczos vector");
     LM_CUDA(s->y.ensure((size_t)n * sizeof(double)), "allocating Lanczos vector");
-    LM_CUDA(s->red.ensure(lmk::lz_red_doubles(n, m_max + 1) * sizeof(double)), "allocating reduction scratch");
+    const size_t step_doubles = lmk::lz_step_doubles(n, m_max + 1);
+    s->lz_one = step_doubles > 0;
+    LM_CUDA(s->red.ensure(std::max(step_doubles, lmk::lz_red_doubles(n, m_max + 1)) * sizeof(double)),
+            "allocating reduction scratch");
     LM_CUDA(s->scal.ensure((size_t)(kScal * (m_max + 3)) * sizeof(double)), "allocating scalars");
     LM_CUDA(s->zbuf.ensure((size_t)m_max * sizeof(double)), "allocating coefficients");
     LM_CUDA(s->cbuf.ensure((size_t)(m_max + 1) * sizeof(double)), "allocating coefficients");
@@ -1144,6 +1156,13 @@ static lm_status sqrt_mdot_body(lm_solver* s, const double* W, uint64_t seed, do
         // the counters must start at zero; the kernels reset them after use
         LM_CUDA(s->lzctr.ensure(ctr_bytes), "allocating counters");
         LM_CUDA(cudaMemsetAsync(s->lzctr.p, 0, s->lzctr.cap, s->stream), "allocating counters");
+    }
+    if (s->lz_one) {
+        // the one-launch iteration's meeting counter (another n: another grid)
+        // and the host's scalars, among them its error words, start at zero;
+        // an earlier call may have left an iteration running ahead
+        LM_CUDA(s->lzmeet.ensure(64), "allocating counters");
+        LM_CUDA(cudaMemsetAsync(s->lzmeet.p, 0, 64, s->stream), "allocating counters");
     }
     if (s->pinned_doubles < (size_t)(kScal * (m_max + 3))) {
         cudaFreeHost(s->pinned);
@@ -1158,6 +1177,7 @@ static lm_status sqrt_mdot_body(lm_solver* s, const double* W, uint64_t seed, do
         LM_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming), "lanczos event");
         s->lz_ev.push_back(e);
     }
+    if (s->lz_one) memset(s->pinned, 0, (size_t)(kScal * (m_max + 3)) * sizeof(double));
     double* V = s->V.as<double>();
     double* w = s->w.as<double>();
     double* scal = s->scal.as<double>();
@@ -1217,14 +1237,23 @@ static lm_status sqrt_mdot_body(lm_solver* s, const double* W, uint64_t seed, do
             if (lm_status st = enqueue_lanczos_iteration(s, k + 1, n, V, w, scal, red, cb, s->lz_ev[k + 1])) return st;
         }
         LM_CUDA(cudaEventSynchronize(s->lz_ev[k]), "lanczos iteration");
+        if (s->lz_one && s->pinned[kScal * k + 3] != 0.0) {
+            cudaStreamSynchronize(s->stream);   // the iteration that runs ahead still writes s->pinned
+            return fail(LM_ERR_TIMEOUT, "a device-side wait expired");
+        }
         const double a_k = s->pinned[kScal * k];
         const double b_k = s->pinned[kScal * k + 1];
-        if (!std::isfinite(a_k) || !std::isfinite(b_k))
+        if (!std::isfinite(a_k) || !std::isfinite(b_k)) {
+            cudaStreamSynchronize(s->stream);
             return fail(LM_ERR_CUDA, "Lanczos produced a non-finite coefficient at iteration %d", k + 1);
+        }
         H.alpha.push_back(a_k);
         const int m = k + 1;
         int ncl = 0;
-        if (H.solve(m, normW, &ncl) != 0) return fail(LM_ERR_NOT_CONVERGED, "tridiagonal eigensolver did not converge");
+        if (H.solve(m, normW, &ncl) != 0) {
+            cudaStreamSynchronize(s->stream);
+            return fail(LM_ERR_NOT_CONVERGED, "tridiagonal eigensolver did not converge");
+        }
         clamped = ncl;
         bool stop = false;
         if (k >= 1) {

@@ -277,6 +277,14 @@ cudaError_t lz_multidot1(const double* V, int m, const double* w, int64_t n, dou
 cudaError_t lz_sub_vc_norm(const double* V, int m, const double* c, double* w, int64_t n, double* red,
                            unsigned* ctr, double* out, cudaStream_t s, const double* cond = nullptr);
 // y = x / nrm[0]
+// One Lanczos iteration after its product in one cooperative launch: alpha,
+// three-term update, Gram-Schmidt, beta (to sc[1]) and row k + 1 of V; the
+// scalars go to host_sc (page-locked, zeroed by the caller).  part: scratch of
+// lz_step_doubles(n, m_max) doubles (0: n or m_max out of its range, use the
+// separate kernels); *ctr: zero, or as the previous lz_step left it.
+size_t lz_step_doubles(int64_t n, int m_max);
+cudaError_t lz_step(double* V, int k, const double* w, int64_t n, double* sc, const double* beta_prev, double* part,
+                    unsigned* ctr, int always_twice, double* host_sc, cudaStream_t s);
 cudaError_t lz_scale(const double* x, const double* nrm, double* y, int64_t n, cudaStream_t s);
 // y = sum_j z[j] v_j
 cudaError_t lz_combine(const double* V, int m, const double* z, double* y, int64_t n, cudaStream_t s);

@@ -7,6 +7,7 @@
 
 #include "lm_internal.cuh"
 #include "pair_common.cuh"
+#include "pdl.cuh"
 
 namespace lmk {
 namespace {
@@ -69,6 +70,7 @@ __global__ void __launch_bounds__(32 * kReduceWarps)
     sym_reduce_kernel(const double* __restrict__ partials, SymGeom g, int64_t block, int C, double c8,
                       const typename V4<R>::type* __restrict__ pos4, int wall, SymOut out, int out_f64) {
     __shared__ double s_p[kReduceWarps][32];
+    pdl_enter();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int64_t e = (int64_t)blockIdx.x * 32 + lane;
     const bool in = e < (int64_t)C * g.N;
@@ -125,10 +127,10 @@ template <typename R>
 cudaError_t launch_sym_reduce(const double* partials, const SymPlan& p, const SymGeom& g, int C, double c8,
                               const void* pos4, int wall, SymOut out, int out_f64, cudaStream_t s) {
     const unsigned blocks = (unsigned)(((int64_t)C * g.N + 31) / 32);
-    sym_reduce_kernel<R><<<blocks, 32 * kReduceWarps, 0, s>>>(partials, g, (int64_t)p.threads * p.ilp, C, c8,
-                                                static_cast<const typename V4<R>::type*>(pos4), wall, out, out_f64);
     count_launches(1);
-    return cudaGetLastError();
+    return launch_pdl(sym_reduce_kernel<R>, dim3(blocks), dim3(32 * kReduceWarps), 0, s, partials, g,
+                      (int64_t)p.threads * p.ilp, C, c8, static_cast<const typename V4<R>::type*>(pos4), wall, out,
+                      out_f64);
 }
 
 template <typename K>
