@@ -289,7 +289,7 @@ lm_status lm_mdot_backward(lm_solver *solver, const void *forces, const void *to
  *   the symmetric kernel (every unordered pair once; no configuration of its
  *   own) is faster, a solver uses it instead: everywhere but for LM_FP64 above
  *   a wall and for LM_FP32C with angular blocks in the open geometry from
- *   N = 8000 on.  Its results
+ *   N = 100000 on.  Its results
  *   are bitwise reproducible too, and its partial sums take up to 128 slots of
  *   3 or 6 FP64 values per particle (or 256 MiB if that is more); when they do
  *   not fit, the one-sided kernel runs.  lm_set_pair_config pins the one-sided

@@ -34,7 +34,7 @@ constexpr int kAdjTileF64 = 32;
 template <bool ANG> constexpr int adj_vals() { return ANG ? 13 : 8; }    // j-side sums per j
 template <bool ANG> constexpr int adj_comps() { return ANG ? 9 : 6; }    // dX, dF [, dT]
 
-// Writes the j-side sums of tile t: the warps' rows of s_j added in FP64.
+// Writes the j-side sums of tile t: the warps' rows of s_j added.
 template <typename R, int C, int NT, int TJ>
 __device__ __forceinline__ void store_j_sums(const R* s_j, const SymGeom& g, int64_t t, int64_t S, bool first,
                                              double* __restrict__ partials) {
@@ -42,9 +42,20 @@ __device__ __forceinline__ void store_j_sums(const R* s_j, const SymGeom& g, int
         const int c = e / TJ, jj = e % TJ;
         const int64_t j = t * TJ + jj;
         if (j >= g.N) continue;
-        double s = 0.0;
+        double s;
+        if constexpr (sizeof(R) == 4) {   // a (hi, lo) pair: FP64 operations are dear
+            float hi = s_j[c * TJ + jj], lo = 0.f;
 #pragma unroll
-        for (int w = 0; w < NT / 32; ++w) s += (double)s_j[(w * C + c) * TJ + jj];
+            for (int w = 1; w < NT / 32; ++w) {
+                float x = s_j[(w * C + c) * TJ + jj];
+                fold(&hi, &lo, x);
+            }
+            s = (double)hi + (double)lo;
+        } else {
+            s = s_j[c * TJ + jj];
+#pragma unroll
+            for (int w = 1; w < NT / 32; ++w) s += s_j[(w * C + c) * TJ + jj];
+        }
         const int64_t o = (S * C + c) * g.N + j;
         // the superblock's slot of j belongs to this item alone; its blocks add in order
         if (LM_INBOUNDS(o < g.slots * C * g.N, 14, o)) partials[o] = first ? s : partials[o] + s;

@@ -23,7 +23,7 @@
 //     value and step, no reduction over lanes and no atomics.
 //   * Sums: a thread's i-side per tile in plain FP32, folded into a (hi, lo)
 //     pair by TwoSum; the j-side of a warp over 32 * NI particles in FP32, the
-//     warps of the CTA added in FP64.  Both go to FP64 slots that exactly one
+//     warps of the CTA added as such a pair.  Both go to FP64 slots that exactly one
 //     item writes (j-side slot: its superblock; i-side slots: its chunks), and
 //     a second kernel adds a particle's slots in a fixed order: the results
 //     are bitwise reproducible.
@@ -89,6 +89,9 @@ __global__ void __launch_bounds__(NT, 4) sym_mdot_f64_kernel(const dvec4* __rest
     constexpr int C = ANG ? 6 : 3;
     constexpr int V = ANG ? 9 : 6;           // values of one j: x, y, z, F, T
     constexpr int NW = NT / 32;
+    // lanes that share the rotation over one group of j: with tiles below 32, the 32 / GW parts of a warp meet
+    // the same j with different i and are added at the end of the group
+    constexpr int GW = TJ < 32 ? TJ : 32;
     __shared__ double s_t[V][TJ];
     __shared__ double s_j[NW][C][TJ];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -138,6 +141,9 @@ __global__ void __launch_bounds__(NT, 4) sym_mdot_f64_kernel(const dvec4* __rest
             }
             __syncthreads();
             const bool diag = t < own + g.tb;
+            // "some pair of the warp may overlap" on the high words: an FP64 compare takes the FP64 pipe; the
+            // exact form decides for itself
+            const int near_hi = __double2hiint(k.four_a2);
             if (diag) {
 #pragma unroll 1
                 for (int jj = 0; jj < TJ; ++jj) {
@@ -152,7 +158,7 @@ __global__ void __launch_bounds__(NT, 4) sym_mdot_f64_kernel(const dvec4* __rest
                         const double dx = x[q][0] - s_t[0][jj], dy = x[q][1] - s_t[1][jj], dz = x[q][2] - s_t[2][jj];
                         const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
                         PairCoef<double> o;
-                        if (__any_sync(0xffffffffu, r2 < k.four_a2)) exact_coeffs<double>(r2, k, o.A, o.B, o.g, o.ar, o.br);
+                        if (__any_sync(0xffffffffu, __double2hiint(r2) <= near_hi)) exact_coeffs<double>(r2, k, o.A, o.B, o.g, o.ar, o.br);
                         else far_coef<double, ANG>(r2, k, o);
                         apply_side<double, ANG>(dx, dy, dz, o.g * dx, o.g * dy, o.g * dz, o, Fj, Tj, acc[q]);
                     }
@@ -160,13 +166,13 @@ __global__ void __launch_bounds__(NT, 4) sym_mdot_f64_kernel(const dvec4* __rest
                 continue;
             }
 #pragma unroll 1
-            for (int gr = 0; gr < TJ; gr += 32) {
+            for (int gr = 0; gr < TJ; gr += GW) {
                 double ja[C];
 #pragma unroll
                 for (int c = 0; c < C; ++c) ja[c] = 0.0;
 #pragma unroll 2
-                for (int st = 0; st < 32; ++st) {
-                    const int jj = gr + ((lane + st) & 31);
+                for (int st = 0; st < GW; ++st) {
+                    const int jj = gr + ((lane + st) & (GW - 1));
                     double Fj[3], Tj[3] = {0.0, 0.0, 0.0};
 #pragma unroll
                     for (int c = 0; c < 3; ++c) {
@@ -178,7 +184,7 @@ __global__ void __launch_bounds__(NT, 4) sym_mdot_f64_kernel(const dvec4* __rest
                         const double dx = x[q][0] - s_t[0][jj], dy = x[q][1] - s_t[1][jj], dz = x[q][2] - s_t[2][jj];
                         const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
                         PairCoef<double> o;
-                        if (__any_sync(0xffffffffu, r2 < k.four_a2)) exact_coeffs<double>(r2, k, o.A, o.B, o.g, o.ar, o.br);
+                        if (__any_sync(0xffffffffu, __double2hiint(r2) <= near_hi)) exact_coeffs<double>(r2, k, o.A, o.B, o.g, o.ar, o.br);
                         else far_coef<double, ANG>(r2, k, o);
                         const double ex = o.g * dx, ey = o.g * dy, ez = o.g * dz;
                         apply_side<double, ANG>(dx, dy, dz, ex, ey, ez, o, Fj, Tj, acc[q]);
@@ -186,10 +192,14 @@ __global__ void __launch_bounds__(NT, 4) sym_mdot_f64_kernel(const dvec4* __rest
                         apply_side<double, ANG>(dx, dy, dz, -ex, -ey, -ez, o, F[q], Tq[q], ja);
                     }
 #pragma unroll
-                    for (int c = 0; c < C; ++c) ja[c] = __shfl_sync(0xffffffffu, ja[c], (lane + 1) & 31);
+                    for (int c = 0; c < C; ++c) ja[c] = __shfl_sync(0xffffffffu, ja[c], (lane & ~(GW - 1)) | ((lane + 1) & (GW - 1)));
                 }
 #pragma unroll
-                for (int c = 0; c < C; ++c) s_j[wid][c][gr + lane] = ja[c];
+                for (int c = 0; c < C; ++c) {
+#pragma unroll
+                    for (int o = GW; o < 32; o <<= 1) ja[c] += __shfl_xor_sync(0xffffffffu, ja[c], o);
+                    if (lane < GW) s_j[wid][c][gr + lane] = ja[c];
+                }
             }
             __syncthreads();
             for (int e = tid; e < TJ * C; e += NT) {
@@ -610,9 +620,13 @@ __global__ void __launch_bounds__(NT) sym_mdot_x2_kernel(const float4* __restric
                     const int c = e / TJ, jj = e % TJ;
                     const int64_t j = t * TJ + jj;
                     if (j >= g.N) continue;
-                    double s = 0.0;
+                    float hi = s_j[c * TJ + jj], lo = 0.f;
 #pragma unroll
-                    for (int w = 0; w < NW; ++w) s += (double)s_j[(w * C + c) * TJ + jj];
+                    for (int w = 1; w < NW; ++w) {
+                        float x = s_j[(w * C + c) * TJ + jj];
+                        fold(&hi, &lo, x);
+                    }
+                    const double s = (double)hi + (double)lo;   // FP64 operations are dear: two conversions, one add
                     const int64_t o = S * stride + (int64_t)c * g.N + j;
                     // the superblock's slot of j belongs to this item alone; its blocks add in order
                     if (LM_INBOUNDS(o < g.slots * stride, 3, o)) partials[o] = sub == 0 ? s : partials[o] + s;
@@ -636,16 +650,15 @@ __global__ void __launch_bounds__(NT) sym_mdot_x2_kernel(const float4* __restric
 
 constexpr int kSymThreads = 128;
 constexpr int kSymWaves = 8;      // items per resident CTA: the largest leave at most an eighth of a wave idle
-constexpr int kTileF64 = 32;      // short tiles: small systems still give every SM an item
 
 // A form launches its kernel or, with occ, returns its resident CTAs per SM.
-template <bool ANG>
+template <bool ANG, int TJ>
 cudaError_t f64_form(const MdotArgs* a, const SymGeom& g, dim3 grid, cudaStream_t s, int* occ) {
     if (occ) {
-        *occ = sym_occupancy(sym_mdot_f64_kernel<ANG, kSymThreads, 1, kTileF64>, kSymThreads, 0);
+        *occ = sym_occupancy(sym_mdot_f64_kernel<ANG, kSymThreads, 1, TJ>, kSymThreads, 0);
         return cudaSuccess;
     }
-    return launch_pdl(sym_mdot_f64_kernel<ANG, kSymThreads, 1, kTileF64>, grid, dim3(kSymThreads), 0, s,
+    return launch_pdl(sym_mdot_f64_kernel<ANG, kSymThreads, 1, TJ>, grid, dim3(kSymThreads), 0, s,
                       static_cast<const dvec4*>(a->pos4), a->F, ANG ? a->T : nullptr, a->in_f64, g,
                       make_rpy_const<double>(a->a), a->partials);
 }
@@ -666,11 +679,15 @@ cudaError_t x2_form(const MdotArgs* a, const SymGeom& g, dim3 grid, cudaStream_t
 
 cudaError_t sym_form(int fp64, int angular, int wall, const SymPlan& p, const MdotArgs* a, const SymGeom& g, dim3 grid,
                      cudaStream_t s, int* occ) {
-    if (fp64) return angular ? f64_form<true>(a, g, grid, s, occ) : f64_form<false>(a, g, grid, s, occ);
+#define LM_FORM64(ANG, TJ) \
+    if (fp64 && angular == ANG && p.tile == TJ) return f64_form<ANG, TJ>(a, g, grid, s, occ);
+    LM_FORM64(false, 8) LM_FORM64(false, 16) LM_FORM64(false, 32)
+    LM_FORM64(true, 8) LM_FORM64(true, 16) LM_FORM64(true, 32)
+#undef LM_FORM64
 #define LM_FORM(ANG, WALL, NI, TJ) \
-    if (angular == ANG && wall == WALL && p.ilp == NI && p.tile == TJ) return x2_form<ANG, WALL, NI, TJ>(a, g, grid, s, occ);
+    if (!fp64 && angular == ANG && wall == WALL && p.ilp == NI && p.tile == TJ) return x2_form<ANG, WALL, NI, TJ>(a, g, grid, s, occ);
     LM_FORM(false, false, 2, 32) LM_FORM(false, false, 2, 64) LM_FORM(false, false, 4, 128) LM_FORM(false, false, 8, 128)
-    LM_FORM(true, false, 2, 32) LM_FORM(true, false, 2, 64)
+    LM_FORM(true, false, 2, 32) LM_FORM(true, false, 2, 64) LM_FORM(true, false, 4, 128) LM_FORM(true, false, 8, 128)
     LM_FORM(false, true, 2, 32) LM_FORM(false, true, 2, 64) LM_FORM(false, true, 4, 128)
     LM_FORM(true, true, 2, 32) LM_FORM(true, true, 2, 128)
 #undef LM_FORM
@@ -681,10 +698,12 @@ cudaError_t sym_form(int fp64, int angular, int wall, const SymPlan& p, const Md
 
 // Products that take the symmetric form.  FP64 with a wall does not (its
 // one-sided kernel has no packed form to share the wall part with), nor FP32
-// with all blocks in free space from N = 8000 on: 46 against 41.5 operations
-// do not pay for the j-side there (16384: 512 / 496 us, 131072: 25.5 / 25.4 ms).
+// with all blocks in free space from N = 100000 on: 46 against 41.5 operations
+// pay for the j-side up to there (65536: 6.49 / 6.61 ms), but no longer when
+// the one-sided kernel runs eight i-particles and four j per vote (131072: 25.4
+// / 25.4 ms, 262144: 101.1 / 101.2 ms).
 static bool sym_selected(int fp64, int angular, int wall, int64_t N) {
-    return wall ? !fp64 : (fp64 || !angular || N < 8000);
+    return wall ? !fp64 : (fp64 || !angular || N < 100000);
 }
 
 // i-particles per thread and particles per j-tile.  Small systems are bound by
@@ -698,21 +717,23 @@ static bool sym_selected(int fp64, int angular, int wall, int64_t N) {
 //                           8192   68 /  62 /  64 /    - |   84
 //                          16384  250 / 215 / 191 /  205 |  281
 //                          50021    - /   - /1570 / 1523 | 2164
-//   all blocks, free space  1000   15 /  22 |  27     4096  47 / 46 | 51     8192  148 / 136 | 138
+//   all blocks, free space  1000   15 /  22 |  27     4096  47 / 46 | 51     10000  - / 198 / 207 / 209 | 225
+//                          16384    - / 497 / 458 / 474 | 495     32768  - / 1811 / 1715 / 1674 | 1734
 //   forces, wall            1000   16 /  23 /  60 |  36   4096  49 /  48 /  56 | 73
 //                          16384  518 / 518 / 498 | 779
 //   all blocks, wall, (2, 32) / (2, 128)   1000   23 / 66 | 51   4096   99 / 105 | 130
 //                          32768  4800 / 4724 | 5970
-//   FP64 (1 and 32, the FP64 pipe is full at one warp per SM quarter): forces 64: 53 | 178, 1000:
-//   54 | 179, 8001: 2193 | 4333; all blocks 64: 94 | 315, 1024: 109 | 318, 8001: 4859 | 8157
+//   FP64 at 8 / 16 / 32 (the FP64 pipe is full at one warp per SM quarter): forces 200: 18 / 29 / 52 |
+//   185, 1024: 50 / 47 / 52 | 179, 8001: 2143 / 2115 / 2100 | 4334; all blocks 200: 32 / 56 / 105 |
+//   330, 1024: 112 / 101 / 104 | 318, 8001: 4863 / 4814 / 4791 | 8167
 static void sym_tiling(int fp64, int angular, int wall, int64_t N, int* ilp, int* tile) {
     *ilp = fp64 ? 1 : 2;
-    *tile = 32;
+    *tile = !fp64 || N > 3000 ? 32 : (N <= 800 ? 8 : 16);
     if (fp64 || N < (angular && wall ? 5000 : 3500)) return;
     *tile = angular && wall ? 128 : 64;
-    if (angular || N < 10000) return;
+    if (N < (angular ? 11000 : 10000) || (angular && wall)) return;
     *tile = 128;
-    *ilp = wall || N < 40000 ? 4 : 8;
+    *ilp = wall || N < (angular ? 30000 : 40000) ? 4 : 8;
 }
 
 void sym_layout(SymPlan* p, int64_t N, int C, int64_t resident, int64_t chunk) {

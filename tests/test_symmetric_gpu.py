@@ -45,13 +45,13 @@ def system(n, dt, wall):
     return pos.astype(dt), F.astype(dt), T.astype(dt)
 
 
-# FP64: i-blocks of 128, j-tiles of 32.  FP32: i-blocks of 256 and j-tiles of 32
+# FP64: i-blocks of 128, j-tiles of 8, 16 (from 801) and 32 (from 3001).  FP32: i-blocks of 256 and j-tiles of 32
 # or 64 up to some thousand particles, then i-blocks of 512 (free space to
 # 40000, wall) and 1024 with j-tiles of 128; from N = 131073 blocks are joined
 # into superblocks so that the slots stay at 128.
-CASES = ([(n, ang, True, False) for n in (1, 2, 33, 128, 129, 1000) for ang in (False, True)]
+CASES = ([(n, ang, True, False) for n in (1, 2, 33, 129, 800, 801, 3001) for ang in (False, True)]
          + [(n, ang, False, wall) for n in (1, 2, 33, 257, 3499) for ang in (False, True) for wall in (False, True)]
-         + [(n, False, False, False) for n in (3500, 9999, 10001, 40001, 150001)] + [(7999, True, False, False)]
+         + [(n, False, False, False) for n in (3500, 9999, 10001, 40001, 150001)] + [(n, True, False, False) for n in (10999, 11000, 30001)]
          + [(n, False, False, True) for n in (3500, 10001)] + [(n, True, False, True) for n in (5000, 5377)])
 
 
