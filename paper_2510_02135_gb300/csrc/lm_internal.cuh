@@ -221,13 +221,14 @@ bool adjoint_config_supported(int fp64, int angular, int threads, int ilp, int u
 int adjoint_ctas_per_sm(int fp64, int angular, int threads, int ilp, int uj);
 
 // Pack N x 3 positions into (x, y, z, 0) and flag non-finite or too large
-// coordinates in *bad (device int, set to 1).
+// coordinates in *bad (device or page-locked host int, set to 1); raw
+// (nullable): a copy of pos.
 cudaError_t launch_pack_positions(const void* pos, int in_f64, int64_t N, void* pos4, int out_f64,
-                                  int* bad, cudaStream_t s);
+                                  int* bad, void* raw, cudaStream_t s);
 // Wall geometry (wall at z = z0): (x, y, max(z - z0, a), f) with the damping
 // factor f = clamp((z - z0) / a, 0, 1).
 cudaError_t launch_pack_wall_positions(const void* pos, int in_f64, int64_t N, double a, double z0, void* pos4,
-                                       int out_f64, int* bad, cudaStream_t s);
+                                       int out_f64, int* bad, void* raw, cudaStream_t s);
 // Random finite differences (wall geometry): pack x + scale W (W: 3N doubles),
 // and write (P - Q) * inv_delta (FP64 grand vectors) to lin / ang.
 cudaError_t launch_displace_pack_wall(const void* pos, int in_f64, const double* W, double scale, int64_t N,

@@ -122,7 +122,7 @@ extern "C" lm_status lm_mdot_noalloc(const float* pos, const float* forces, cons
     if (lmk::mdot_effective_splits(N, threads, splits) > max_splits)
         return noalloc_fail(LM_ERR_INVALID_ARG, "scratch too small for N = %lld", (long long)N);
 
-    e = lmk::launch_pack_positions(pos, 0, N, pos4, 0, flag, stream);
+    e = lmk::launch_pack_positions(pos, 0, N, pos4, 0, flag, nullptr, stream);
     if (e != cudaSuccess) return noalloc_fail(LM_ERR_CUDA, "packing positions: %s", cudaGetErrorString(e));
     if (forces == nullptr && torques == nullptr) {
         e = cudaMemsetAsync(lin_out, 0, (size_t)N * 3 * sizeof(float), stream);

@@ -38,6 +38,27 @@ __device__ __forceinline__ R load_elem(const void* p, int in_f64, int64_t idx) {
     return in_f64 ? (R)(static_cast<const double*>(p)[idx]) : (R)(static_cast<const float*>(p)[idx]);
 }
 
+// Position i of the caller's N x 3 array; raw (nullable): a copy of the array.
+__device__ __forceinline__ void load_raw_position(const void* pos, int f64, int64_t i, void* raw, double* x, double* y,
+                                                  double* z) {
+    if (f64) {
+        const double* p = static_cast<const double*>(pos) + 3 * i;
+        *x = p[0]; *y = p[1]; *z = p[2];
+        if (raw) {
+            double* q = static_cast<double*>(raw) + 3 * i;
+            q[0] = *x; q[1] = *y; q[2] = *z;
+        }
+    } else {
+        const float* p = static_cast<const float*>(pos) + 3 * i;
+        const float a = p[0], b = p[1], c = p[2];
+        *x = a; *y = b; *z = c;
+        if (raw) {
+            float* q = static_cast<float*>(raw) + 3 * i;
+            q[0] = a; q[1] = b; q[2] = c;
+        }
+    }
+}
+
 // Exact pair coefficients (both branches) for one pair.
 template <typename R>
 __device__ __forceinline__ void exact_coeffs(R r2, const RpyConst<R>& k, R& A, R& B, R& g, R& ar, R& br) {

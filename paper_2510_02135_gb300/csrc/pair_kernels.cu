@@ -645,20 +645,15 @@ cudaError_t launch_mdot(const MdotArgs& a, cudaStream_t s) {
 namespace {
 template <typename RO>
 __global__ void pack_positions_kernel(const void* __restrict__ pos, int in_f64, int64_t N,
-                                      typename V4<RO>::type* __restrict__ out, int* __restrict__ bad) {
+                                      typename V4<RO>::type* __restrict__ out, int* __restrict__ bad,
+                                      void* __restrict__ raw) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     double x, y, z;
-    if (in_f64) {
-        const double* p = static_cast<const double*>(pos);
-        x = p[3 * i]; y = p[3 * i + 1]; z = p[3 * i + 2];
-    } else {
-        const float* p = static_cast<const float*>(pos);
-        x = p[3 * i]; y = p[3 * i + 1]; z = p[3 * i + 2];
-    }
+    load_raw_position(pos, in_f64, i, raw, &x, &y, &z);
     const double m = kMaxAbsCoord;
     // written as a negated "inside" test so that NaN counts as bad
-    if (!(fabs(x) <= m && fabs(y) <= m && fabs(z) <= m)) atomicExch(bad, 1);
+    if (!(fabs(x) <= m && fabs(y) <= m && fabs(z) <= m)) *(volatile int*)bad = 1;
     typename V4<RO>::type v;
     v.x = (RO)x; v.y = (RO)y; v.z = (RO)z; v.w = (RO)0;
     out[i] = v;
@@ -666,13 +661,13 @@ __global__ void pack_positions_kernel(const void* __restrict__ pos, int in_f64, 
 }  // namespace
 
 cudaError_t launch_pack_positions(const void* pos, int in_f64, int64_t N, void* pos4, int out_f64, int* bad,
-                                  cudaStream_t s) {
+                                  void* raw, cudaStream_t s) {
     if (N <= 0) return cudaSuccess;
     const unsigned blocks = (unsigned)((N + 255) / 256);
     if (out_f64)
-        pack_positions_kernel<double><<<blocks, 256, 0, s>>>(pos, in_f64, N, static_cast<dvec4*>(pos4), bad);
+        pack_positions_kernel<double><<<blocks, 256, 0, s>>>(pos, in_f64, N, static_cast<dvec4*>(pos4), bad, raw);
     else
-        pack_positions_kernel<float><<<blocks, 256, 0, s>>>(pos, in_f64, N, static_cast<float4*>(pos4), bad);
+        pack_positions_kernel<float><<<blocks, 256, 0, s>>>(pos, in_f64, N, static_cast<float4*>(pos4), bad, raw);
     count_launches(1);
     return cudaGetLastError();
 }

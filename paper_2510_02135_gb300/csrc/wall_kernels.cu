@@ -688,19 +688,14 @@ cudaError_t launch_wall_mdot(const MdotArgs& a, cudaStream_t s) {
 namespace {
 template <typename RO>
 __global__ void pack_wall_positions_kernel(const void* __restrict__ pos, int in_f64, int64_t N, double a, double z0,
-                                           typename V4<RO>::type* __restrict__ out, int* __restrict__ bad) {
+                                           typename V4<RO>::type* __restrict__ out, int* __restrict__ bad,
+                                           void* __restrict__ raw) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     double x, y, z;
-    if (in_f64) {
-        const double* p = static_cast<const double*>(pos);
-        x = p[3 * i]; y = p[3 * i + 1]; z = p[3 * i + 2];
-    } else {
-        const float* p = static_cast<const float*>(pos);
-        x = p[3 * i]; y = p[3 * i + 1]; z = p[3 * i + 2];
-    }
+    load_raw_position(pos, in_f64, i, raw, &x, &y, &z);
     const double m = kMaxAbsCoord;
-    if (!(fabs(x) <= m && fabs(y) <= m && fabs(z) <= m)) atomicExch(bad, 1);
+    if (!(fabs(x) <= m && fabs(y) <= m && fabs(z) <= m)) *(volatile int*)bad = 1;
     z -= z0;   // height above the wall
     double f = z / a;
     f = f > 0.0 ? (f < 1.0 ? f : 1.0) : 0.0;
@@ -840,15 +835,15 @@ cudaError_t launch_rfd_difference(const double* P, const double* Q, double inv_d
 }
 
 cudaError_t launch_pack_wall_positions(const void* pos, int in_f64, int64_t N, double a, double z0, void* pos4,
-                                       int out_f64, int* bad, cudaStream_t s) {
+                                       int out_f64, int* bad, void* raw, cudaStream_t s) {
     if (N <= 0) return cudaSuccess;
     const unsigned blocks = (unsigned)((N + 255) / 256);
     if (out_f64)
         pack_wall_positions_kernel<double><<<blocks, 256, 0, s>>>(pos, in_f64, N, a, z0, static_cast<dvec4*>(pos4),
-                                                                   bad);
+                                                                   bad, raw);
     else
         pack_wall_positions_kernel<float><<<blocks, 256, 0, s>>>(pos, in_f64, N, a, z0, static_cast<float4*>(pos4),
-                                                                  bad);
+                                                                  bad, raw);
     count_launches(1);
     return cudaGetLastError();
 }
