@@ -440,7 +440,7 @@ __global__ void __launch_bounds__(NT, MINB) rpy_adjoint_x2_kernel(const float4* 
 #pragma unroll
                     for (int pp = 0; pp < NP; ++pp) {
                         const float2 ddx = dx[u][pp], ddy = dy[u][pp], ddz = dz[u][pp];
-                        const float2 invr = make_float2(rsqrtf(r2[u][pp].x), rsqrtf(r2[u][pp].y));
+                        const float2 invr = make_float2(rsq_far(r2[u][pp].x), rsq_far(r2[u][pp].y));
                         const float2 invr2 = mul2(invr, invr);
                         const float2 invr3 = mul2(invr2, invr);
                         const float2 invr5 = mul2(invr3, invr2);

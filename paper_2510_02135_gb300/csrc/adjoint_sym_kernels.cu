@@ -565,7 +565,7 @@ __global__ void __launch_bounds__(NT) adj_sym_x2_kernel(const float4* __restrict
                     PCoef2 c;
                     float2 gg = bc2(0.f);
                     if (!near) {
-                        const float2 invr = make_float2(rsqrtf(r2[p].x), rsqrtf(r2[p].y));
+                        const float2 invr = make_float2(rsq_far(r2[p].x), rsq_far(r2[p].y));
                         const float2 invr2 = mul2(invr, invr);
                         const float2 invr3 = mul2(invr2, invr);
                         const float2 invr5 = mul2(invr3, invr2);

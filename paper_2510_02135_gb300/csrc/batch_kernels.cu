@@ -38,6 +38,7 @@
 #include <cstdint>
 
 #include "lm_internal.cuh"
+#include "pair_common.cuh"
 #include "philox.cuh"
 #include "tridiag.cuh"
 #include "tridiag_dev.cuh"
@@ -250,7 +251,7 @@ __device__ void pair_item(const BatchParams& P, int s, int i0, int jb, int je, c
                     A = make_float2(a_[0], a_[1]);
                     B = make_float2(b_[0], b_[1]);
                 } else {
-                    const float2 invr = make_float2(rsqrtf(r2[u][q].x), rsqrtf(r2[u][q].y));
+                    const float2 invr = make_float2(rsq_far(r2[u][q].x), rsq_far(r2[u][q].y));
                     const float2 invr2 = __fmul2_rn(invr, invr);
                     const float2 invr3 = __fmul2_rn(invr2, invr);
                     A = __ffma2_rn(K1, invr3, invr);

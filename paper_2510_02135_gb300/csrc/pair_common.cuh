@@ -20,11 +20,17 @@ template <> struct V4<double> { using type = lmk::dvec4; };
 __device__ __forceinline__ float rsq(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double rsq(double x) { return 1.0 / sqrt(x); }
 
-// 1 / sqrt(x) for normal x > 0 in the far field.  FP64: the instruction's
+// 1 / sqrt(x) for normal x > 0 in the far field.  FP32: the instruction itself
+// (rsqrtf adds a test and two predicated multiplications for subnormal x; a
+// third of a pair's scalar instructions).  FP64: the instruction's
 // estimate (relative error d, 2^-20 or better) and one third-order step,
 // y (1 + e (1/2 + 3 e / 8)) with e = 1 - x y^2, which leaves (5/2) d^3 and the
 // rounding: 5 FP64 operations against about 20 for 1 / sqrt.
-__device__ __forceinline__ float rsq_far(float x) { return rsqrtf(x); }
+__device__ __forceinline__ float rsq_far(float x) {
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
 __device__ __forceinline__ double rsq_far(double x) {
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
@@ -98,7 +104,7 @@ template <typename R, bool ANG>
 __device__ __forceinline__ void pair_far(R dx, R dy, R dz, R r2, const typename V4<R>::type& f,
                                          const typename V4<R>::type& h, const RpyConst<R>& k,
                                          Acc<R, ANG>& acc) {
-    const R invr = rsq(r2);
+    const R invr = rsq_far(r2);
     const R invr2 = invr * invr;
     const R invr3 = invr2 * invr;
     const R A = fma(k.K1, invr3, invr);

@@ -324,7 +324,7 @@ __device__ __forceinline__ void x2_segment(const float4* __restrict__ pos4, cons
                 const float4 w1 = s_t[1 * NT + jj + u];
                 const float2 fx = bc2(w0.w), fy = bc2(w1.x), fz = bc2(w1.y);
                 const float2 ddx = dx[u][p], ddy = dy[u][p], ddz = dz[u][p];
-                const float2 invr = make_float2(rsqrtf(r2[u][p].x), rsqrtf(r2[u][p].y));
+                const float2 invr = make_float2(rsq_far(r2[u][p].x), rsq_far(r2[u][p].y));
                 const float2 invr2 = mul2(invr, invr);
                 const float2 invr3 = mul2(invr2, invr);
                 const float2 A = fma2(K1, invr3, invr);

@@ -266,7 +266,7 @@ __device__ __forceinline__ JVal sym_load_j(const float4* __restrict__ s_t, int j
 template <bool ANG, bool SYM>
 __device__ __forceinline__ void sym_far2(float2 dx, float2 dy, float2 dz, float2 r2, float2 K1, float2 nK2,
                                          const JVal& j, const float2* F, const float2* T, float2* acc, float2* ja) {
-    const float2 invr = make_float2(rsqrtf(r2.x), rsqrtf(r2.y));
+    const float2 invr = make_float2(rsq_far(r2.x), rsq_far(r2.y));
     const float2 invr2 = mul2(invr, invr);
     const float2 g = mul2(invr2, invr);
     const float2 A = fma2(K1, g, invr);
@@ -349,7 +349,7 @@ __device__ __forceinline__ void sym_wall2(float2 Rx, float2 Ry, float2 zi, float
                                           const float2* T, float2* acc, float2* ja) {
     const float2 Rz = add2(zi, j.z);
     const float2 r2 = fma2(Rx, Rx, fma2(Ry, Ry, mul2(Rz, Rz)));
-    const float2 u = make_float2(rsqrtf(r2.x), rsqrtf(r2.y));
+    const float2 u = make_float2(rsq_far(r2.x), rsq_far(r2.y));
     const float2 ex = mul2(Rx, u), ey = mul2(Ry, u), c = mul2(Rz, u);
     const float2 H = mul2(j.z, u);
     const float2 al = mul2(mul2(a2, u), u);

@@ -45,7 +45,7 @@ namespace {
 template <typename R, bool ANG>
 __device__ __forceinline__ void wall_pair(R Rx, R Ry, R Rz, R hj, const typename V4<R>::type& f,
                                           const typename V4<R>::type& th, R a2, Acc<R, ANG>& acc) {
-    const R u = rsq(fma(Rx, Rx, fma(Ry, Ry, Rz * Rz)));
+    const R u = rsq_far(fma(Rx, Rx, fma(Ry, Ry, Rz * Rz)));
     const R ex = Rx * u, ey = Ry * u, c = Rz * u;
     const R H = hj * u;
     const R al = a2 * u * u;
@@ -251,7 +251,7 @@ __device__ __forceinline__ void wall_pair2(float2 Rx, float2 Ry, float2 zi, floa
                                            float2* acc) {
     const float2 Rz = add2(zi, zj);
     const float2 r2 = fma2(Rx, Rx, fma2(Ry, Ry, mul2(Rz, Rz)));
-    const float2 u = make_float2(rsqrtf(r2.x), rsqrtf(r2.y));
+    const float2 u = make_float2(rsq_far(r2.x), rsq_far(r2.y));
     const float2 ex = mul2(Rx, u), ey = mul2(Ry, u), c = mul2(Rz, u);
     const float2 H = mul2(zj, u);
     const float2 al = mul2(mul2(a2, u), u);
@@ -440,7 +440,7 @@ __global__ void __launch_bounds__(NT) rpy_wall_x2_kernel(const float4* __restric
             }
             // open-space far-field pair of slot p (two i-particles against j)
             auto far_slot = [&](int p) {
-                const float2 invr = make_float2(rsqrtf(r2[p].x), rsqrtf(r2[p].y));
+                const float2 invr = make_float2(rsq_far(r2[p].x), rsq_far(r2[p].y));
                 const float2 invr2 = mul2(invr, invr);
                 const float2 invr3 = mul2(invr2, invr);
                 const float2 A = fma2(K1, invr3, invr);
