@@ -443,6 +443,18 @@ void ensure_config(lm_solver* s) {
     s->cfg_N = s->N;
 }
 
+// Whether the partial sums have, or may get, `bytes`: an allocation would end a
+// stream capture, and the one-sided forms of the smallest systems need none.
+bool can_allocate(const lm_solver* s, size_t bytes) {
+    if (s->partials.p != nullptr && bytes <= s->partials.cap) return true;
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s->stream, &st) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return st == cudaStreamCaptureStatusNone;
+}
+
 // Whether the product takes the symmetric form: its rule selects this (precision,
 // blocks, geometry, N), no one-sided kernel is pinned and its partial sums fit
 // the device (else the one-sided form, which needs fewer, serves).
@@ -455,6 +467,7 @@ bool sym_form(lm_solver* s) {
     if (!s->sym_ok) return false;
     const size_t bytes =
         (size_t)s->sym.slots * lmk::mdot_partial_components(s->angular) * (size_t)s->N * sizeof(double);
+    if (!can_allocate(s, bytes)) return false;
     if (s->partials.ensure(bytes) != cudaSuccess) {
         cudaGetLastError();
         s->sym_ok = false;
@@ -609,7 +622,7 @@ lm_status run_adjoint(lm_solver* s, const void* F, const void* T, const void* G,
         }
         const size_t pb = (size_t)s->adj_sym.slots * lmk::adjoint_partial_components(s->angular) * (size_t)s->N *
                           sizeof(double);
-        if (s->partials.ensure(pb) != cudaSuccess) {
+        if (!can_allocate(s, pb) || s->partials.ensure(pb) != cudaSuccess) {
             // no room for the slots: the one-sided form, which needs fewer
             cudaGetLastError();
             return run_adjoint(s, F, T, G, H, dX, dF, dT, one_sided_adjoint_config(s));

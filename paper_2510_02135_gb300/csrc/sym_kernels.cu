@@ -7,8 +7,8 @@
 //   pair work (FMA-lane operations per ordered pair)     one-sided  symmetric
 //     free space, forces only                                21        15.5
 //     free space, all blocks                                 46        41.5
-//     single wall, forces only                               66        44
-//     single wall, all blocks                               150       110
+//     single wall, forces only                               80        52
+//     single wall, all blocks                               170       134
 //
 // Schedule:
 //   * Item (S, c): the i-blocks of superblock S (m blocks of NT * NI
@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(NT, 4) sym_mdot_f64_kernel(const dvec4* __rest
     __shared__ double s_j[NW][C][TJ];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const double pad = kPadCoord;
-    pdl_enter();
+    pdl_enter();   // the slot sums may be launched from here on
     SymItem it;
     if (!sym_item(g, &it)) return;
     const int64_t S = it.S, t0 = it.t0, t1 = it.t1;
@@ -454,7 +454,7 @@ __global__ void __launch_bounds__(NT) sym_mdot_x2_kernel(const float4* __restric
     float* s_j = s_lo + C * NI * NT;                            // [warp][c][jj]
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const float pad = (float)kPadCoord;
-    pdl_enter();
+    pdl_enter();   // the slot sums may be launched from here on
     SymItem it;
     if (!sym_item(g, &it)) return;
     const int64_t S = it.S, t0 = it.t0, t1 = it.t1;
@@ -658,9 +658,10 @@ cudaError_t f64_form(const MdotArgs* a, const SymGeom& g, dim3 grid, cudaStream_
         *occ = sym_occupancy(sym_mdot_f64_kernel<ANG, kSymThreads, 1, TJ>, kSymThreads, 0);
         return cudaSuccess;
     }
-    return launch_pdl(sym_mdot_f64_kernel<ANG, kSymThreads, 1, TJ>, grid, dim3(kSymThreads), 0, s,
-                      static_cast<const dvec4*>(a->pos4), a->F, ANG ? a->T : nullptr, a->in_f64, g,
-                      make_rpy_const<double>(a->a), a->partials);
+    sym_mdot_f64_kernel<ANG, kSymThreads, 1, TJ><<<grid, kSymThreads, 0, s>>>(
+        static_cast<const dvec4*>(a->pos4), a->F, ANG ? a->T : nullptr, a->in_f64, g, make_rpy_const<double>(a->a),
+        a->partials);
+    return cudaGetLastError();
 }
 
 template <bool ANG, bool WALL, int NI, int TJ>
@@ -672,9 +673,12 @@ cudaError_t x2_form(const MdotArgs* a, const SymGeom& g, dim3 grid, cudaStream_t
     }
     static std::atomic<unsigned long long> attr_devs{0};  // devices whose limit is raised
     if (cudaError_t e = smem_attr_once(attr_devs, sym_mdot_x2_kernel<ANG, WALL, kSymThreads, NI, TJ>, dyn)) return e;
-    return launch_pdl(sym_mdot_x2_kernel<ANG, WALL, kSymThreads, NI, TJ>, grid, dim3(kSymThreads), dyn, s,
-                      static_cast<const float4*>(a->pos4), a->F, ANG ? a->T : nullptr, a->in_f64, g,
-                      make_rpy_const<float>(a->a), (float)(a->a * a->a), a->partials);
+    // a plain launch: CTAs that start among the last ones of the kernel before are spread unevenly over the SMs, and
+    // a small product lasts as long as its fullest SM (wall, N = 4096: 64 us against 48)
+    sym_mdot_x2_kernel<ANG, WALL, kSymThreads, NI, TJ><<<grid, kSymThreads, dyn, s>>>(
+        static_cast<const float4*>(a->pos4), a->F, ANG ? a->T : nullptr, a->in_f64, g, make_rpy_const<float>(a->a),
+        (float)(a->a * a->a), a->partials);
+    return cudaGetLastError();
 }
 
 cudaError_t sym_form(int fp64, int angular, int wall, const SymPlan& p, const MdotArgs* a, const SymGeom& g, dim3 grid,
