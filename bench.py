@@ -327,7 +327,9 @@ def hotpath_leg(workload, steps, warmup, dist, local, *, pair_config=None, autot
     achieved = prof["pair_flops"] / (prof["pair_ms"] / 1e3) / 1e12 if prof["pair_ms"] > 0 else None
     roofline = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": (achieved / peak) if achieved else None, "traffic": profile_traffic(workload),
-                "kernel": ("rpy_mdot_x2_kernel (forward pair kernel, packed FP32, all four blocks)" if cfg["packed"]
+                "kernel": ("sym_mdot_x2_kernel (symmetric pair kernel, packed FP32, all four blocks; every unordered "
+                           "pair once, flops counted per ordered pair)" if n < 100_000 and not pair_config
+                           else "rpy_mdot_x2_kernel (forward pair kernel, packed FP32, all four blocks)" if cfg["packed"]
                            else "rpy_mdot_kernel (forward pair kernel, scalar FP32, all four blocks)"),
                 "flops_per_pair": FLOPS_PER_PAIR_6N, "pairs_per_launch": float(n) * n,
                 "pair_launches": prof["pair_launches"],

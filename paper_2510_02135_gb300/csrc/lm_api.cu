@@ -347,7 +347,8 @@ lm_pair_config default_config(const lm_solver* s, int64_t N) {
     c.ilp = s->fp64 ? (s->angular ? 1 : 2) : (s->angular ? 4 : 8);
     c.packed = s->fp64 ? 0 : 1;
     if (!s->fp64 && s->angular && !s->wall && N >= 100000) {
-        // many i-blocks: eight i-particles per thread and four j per vote (131072: 25.4 / 25.7 ms, 524288: 403 / 412)
+        // many i-blocks: eight i-particles per thread and four j per vote (131072: 25.4 / 25.7 ms, 524288: 403 / 412
+        // with rsqrtf; 23.8 and 376 since)
         c.ilp = 8;
         c.packed = 4;
     }
@@ -566,7 +567,8 @@ lm_pair_config one_sided_adjoint_config(const lm_solver* s) {
 // 6.61 / 6.27 / 8.43 ms; with angular blocks 1024 64 / 103 / 177 us, 4096 103 /
 // 109 / 174, 16384 1156 / 1061 / 1776, 65536 17.1 / 15.5 / 27.0 ms.  FP64 (ilp
 // 1): 1024 0.12 / 1.17 ms, 8001 4.97 / 8.48 ms; with angular blocks 4096 3.18 /
-// 5.91 ms.
+// 5.91 ms.  (With rsqrtf; the symmetric ones since: 4096 48 us, 8192 123, 65536
+// 5.88 ms; with angular blocks 1024 60 us, 4096 95, 16384 1022, 65536 15.3 ms.)
 lm_pair_config default_adjoint_config(const lm_solver* s) {
     if (s->fp64) return lm_pair_config{128, 1, 0, 3};
     const int ilp = s->N <= 10000 ? 2 : 4;

@@ -705,7 +705,8 @@ cudaError_t sym_form(int fp64, int angular, int wall, const SymPlan& p, const Md
 // with all blocks in free space from N = 100000 on: 46 against 41.5 operations
 // pay for the j-side up to there (65536: 6.49 / 6.61 ms), but no longer when
 // the one-sided kernel runs eight i-particles and four j per vote (131072: 25.4
-// / 25.4 ms, 262144: 101.1 / 101.2 ms).
+// / 25.4 ms, 262144: 101.1 / 101.2 ms; 65536 since the far field takes the bare
+// reciprocal root: 6.31 / 6.20 ms, 50000 3.69 / 3.97, 99000 14.2 / 15.6).
 static bool sym_selected(int fp64, int angular, int wall, int64_t N) {
     return wall ? !fp64 : (fp64 || !angular || N < 100000);
 }
@@ -713,8 +714,10 @@ static bool sym_selected(int fp64, int angular, int wall, int64_t N) {
 // i-particles per thread and particles per j-tile.  Small systems are bound by
 // the latency of one item, so short tiles and few i-particles make more and
 // shorter items; large ones by the FMA pipe, where more i-particles share a
-// j-value and its shuffles.  Device time of a product on GB300, us, symmetric
-// at (2, 32) / (2, 64) / (4, 128) / (8, 128) and one-sided with its default:
+// j-value and its shuffles.  Device time of a product on GB300, us (taken with
+// rsqrtf; the bare instruction took 4-7% off either side since: 50021 1422,
+// 32768 all blocks 1628, wall 1780, wall with all blocks 4610), symmetric at
+// (2, 32) / (2, 64) / (4, 128) / (8, 128) and one-sided with its default:
 //   forces, free space   N = 100   11 /  15 /  28 /    - |   22
 //                           1000   13 /  16 /  31 /    - |   24
 //                           4096   26 /  24 /  31 /    - |   33
