@@ -85,7 +85,15 @@ lm_status lm_create(lm_solver **out, const char *px, const char *py, const char 
 /* lm_destroy -- frees the solver and all its device memory.  NULL is allowed. */
 lm_status lm_destroy(lm_solver *solver);
 
-/* lm_set_stream -- change the CUDA stream used by later calls. */
+/*
+ * lm_set_stream -- change the CUDA stream used by later calls.  The calls of a
+ * solver share its scratch memory, except that lm_mdot and lm_mdot_backward
+ * each have partial sums of their own: calls of one kind on different streams
+ * are to be ordered by the caller.  Scratch is allocated by the first call of
+ * its kind at a given N, kept, and replaced when a later call needs more; a
+ * call that is captured in a CUDA graph wants one such call before the
+ * capture, and none that needs more while the graph is in use.
+ */
 lm_status lm_set_stream(lm_solver *solver, void *cuda_stream);
 
 /*

@@ -153,7 +153,9 @@ struct lm_solver {
     bool has_pos = false;
 
     DBuf pos4;
-    DBuf partials;
+    // partial sums of the product and of the adjoint: apart, so that a product captured in a graph or running on
+    // another stream keeps its buffer when a gradient is taken
+    DBuf partials, adj_partials;
     DBuf in_stage[4];
     DBuf out_stage[3];
     DBuf flag;
@@ -176,6 +178,7 @@ struct lm_solver {
     // plan of the symmetric adjoint, for (N, threads, ilp, splits, packed)
     lmk::SymPlan adj_sym{};
     std::array<int64_t, 5> adj_sym_key{{-1, 0, 0, 0, 0}};
+    bool adj_sym_ok = false;   // false: its slots did not fit
     double* pinned = nullptr;  // host scalar read-back
     size_t pinned_doubles = 0;
 
@@ -211,7 +214,7 @@ struct lm_solver {
     size_t vprof_used = 0;
 
     ~lm_solver() {
-        DBuf* all[] = {&pos4, &partials, &in_stage[0], &in_stage[1], &in_stage[2], &in_stage[3],
+        DBuf* all[] = {&pos4, &partials, &adj_partials, &in_stage[0], &in_stage[1], &in_stage[2], &in_stage[3],
                        &out_stage[0], &out_stage[1], &out_stage[2], &flag, &tune_in, &tune_out,
                        &pos_raw, &rfd_pos4, &rfd_W, &rfd_P, &rfd_Q, &ab_u, &ab_d, &ab_y, &ab_x, &pc_p, &pc_q, &pc_t, &lzctr, &lzmeet,
                        &V, &w, &y, &red, &scal, &zbuf, &cbuf, &Wbuf};
@@ -446,8 +449,8 @@ void ensure_config(lm_solver* s) {
 
 // Whether the partial sums have, or may get, `bytes`: an allocation would end a
 // stream capture, and the one-sided forms of the smallest systems need none.
-bool can_allocate(const lm_solver* s, size_t bytes) {
-    if (s->partials.p != nullptr && bytes <= s->partials.cap) return true;
+bool can_allocate(const lm_solver* s, const DBuf& partials, size_t bytes) {
+    if (partials.p != nullptr && bytes <= partials.cap) return true;
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s->stream, &st) != cudaSuccess) {
         cudaGetLastError();
@@ -468,7 +471,7 @@ bool sym_form(lm_solver* s) {
     if (!s->sym_ok) return false;
     const size_t bytes =
         (size_t)s->sym.slots * lmk::mdot_partial_components(s->angular) * (size_t)s->N * sizeof(double);
-    if (!can_allocate(s, bytes)) return false;
+    if (!can_allocate(s, s->partials, bytes)) return false;
     if (s->partials.ensure(bytes) != cudaSuccess) {
         cudaGetLastError();
         s->sym_ok = false;
@@ -621,24 +624,27 @@ lm_status run_adjoint(lm_solver* s, const void* F, const void* T, const void* G,
             lmk::sym_layout(&s->adj_sym, s->N, lmk::adjoint_partial_components(s->angular),
                             (int64_t)occ * s->sm_count, chunk);
             s->adj_sym_key = key;
+            s->adj_sym_ok = true;
         }
         const size_t pb = (size_t)s->adj_sym.slots * lmk::adjoint_partial_components(s->angular) * (size_t)s->N *
                           sizeof(double);
-        if (!can_allocate(s, pb) || s->partials.ensure(pb) != cudaSuccess) {
-            // no room for the slots: the one-sided form, which needs fewer
+        bool room = s->adj_sym_ok && can_allocate(s, s->adj_partials, pb);
+        if (room && s->adj_partials.ensure(pb) != cudaSuccess) {
             cudaGetLastError();
-            return run_adjoint(s, F, T, G, H, dX, dF, dT, one_sided_adjoint_config(s));
+            room = s->adj_sym_ok = false;
         }
+        // no room for the slots: the one-sided form, which needs fewer
+        if (!room) return run_adjoint(s, F, T, G, H, dX, dF, dT, one_sided_adjoint_config(s));
         a.sym = s->adj_sym;
-        a.partials = s->partials.as<double>();
+        a.partials = s->adj_partials.as<double>();
         LM_CUDA(lmk::launch_adjoint(a, s->stream), "adjoint kernel");
         return LM_OK;
     }
     const int64_t se = lmk::mdot_effective_splits(s->N, a.threads, a.splits);
     if (se > 1) {
         const size_t pb = (size_t)se * lmk::adjoint_partial_components(s->angular) * (size_t)s->N * sizeof(double);
-        LM_CUDA(s->partials.ensure(pb), "allocating split partial sums");
-        a.partials = s->partials.as<double>();
+        LM_CUDA(s->adj_partials.ensure(pb), "allocating split partial sums");
+        a.partials = s->adj_partials.as<double>();
     }
     LM_CUDA(lmk::launch_adjoint(a, s->stream), "adjoint kernel");
     return LM_OK;
