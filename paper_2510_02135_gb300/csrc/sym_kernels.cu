@@ -39,8 +39,8 @@ namespace {
 // ---------------------------------------------------------------------------
 // Scalar form (FP64).  The FP64 pipe takes one warp instruction per 64 cycles
 // and SM quarter, so a warp per quarter saturates it and the time is the
-// number of FP64 instructions: 38 (forces only) or 85 (all blocks) per
-// unordered pair.
+// number of FP64 operations: 31 (forces only) or 80 (all blocks) and a
+// reciprocal square root per unordered pair.
 // ---------------------------------------------------------------------------
 template <typename R>
 struct PairCoef {
