@@ -19,6 +19,7 @@
 #include <vector>
 
 #include "../../include/lm.h"
+#include "host_scalars.h"
 #include "lm_internal.cuh"
 #include "lm_runtime.cuh"
 #include "tridiag.cuh"
@@ -227,6 +228,12 @@ struct lm_solver {
 };
 
 namespace {
+
+cudaError_t grow_pinned(lm_solver* s, size_t doubles) {
+    return lmk::grow_host_doubles<cudaError_t>(
+        &s->pinned, &s->pinned_doubles, doubles, [](void** p, size_t bytes) { return cudaMallocHost(p, bytes); },
+        [](void* p) { return cudaFreeHost(p); });
+}
 
 size_t elem_size(const lm_solver* s) { return s->fp64 ? sizeof(double) : sizeof(float); }
 
@@ -764,10 +771,7 @@ lm_status lm_create(lm_solver** out, const char* px, const char* py, const char*
     cudaError_t e = cudaGetDevice(&s->device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&s->sm_count, cudaDevAttrMultiProcessorCount, s->device);
     if (e == cudaSuccess) e = s->flag.ensure(64);
-    if (e == cudaSuccess) {
-        s->pinned_doubles = 64;
-        e = cudaMallocHost(reinterpret_cast<void**>(&s->pinned), s->pinned_doubles * sizeof(double));
-    }
+    if (e == cudaSuccess) e = grow_pinned(s, 64);
     if (e != cudaSuccess) {
         lm_status st = cuda_fail(e, "lm_create");
         delete s;
@@ -1190,14 +1194,7 @@ static lm_status sqrt_mdot_body(lm_solver* s, const double* W, uint64_t seed, do
         LM_CUDA(s->lzmeet.ensure(64), "allocating counters");
         LM_CUDA(cudaMemsetAsync(s->lzmeet.p, 0, 64, s->stream), "allocating counters");
     }
-    if (s->pinned_doubles < (size_t)(kScal * (m_max + 3))) {
-        cudaFreeHost(s->pinned);
-        s->pinned = nullptr;
-        s->pinned_doubles = 0;
-        LM_CUDA(cudaMallocHost(reinterpret_cast<void**>(&s->pinned), (size_t)(kScal * (m_max + 3)) * sizeof(double)),
-                "allocating pinned scalars");
-        s->pinned_doubles = (size_t)(kScal * (m_max + 3));
-    }
+    LM_CUDA(grow_pinned(s, (size_t)kScal * (m_max + 3)), "allocating pinned scalars");
     while (s->lz_ev.size() < (size_t)(m_max + 1)) {
         cudaEvent_t e;
         LM_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming), "lanczos event");
