@@ -8,6 +8,8 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <cstdlib>
+#include <cstring>
 
 #include "lm_internal.cuh"
 #include "pdl.cuh"
@@ -355,16 +357,21 @@ __global__ void sub_vc_norm_kernel(const double* __restrict__ V, int m, const do
 constexpr int kStepThreads = 256;
 constexpr long long kStepSpinCycles = 4000000000ll;   // about 2 s
 
-__device__ __forceinline__ bool step_meet(unsigned* ctr, unsigned* target) {
+struct StepMeet {
+    unsigned* ctr;
+    unsigned target, arrivals;   // thread 0's: arrivals that end the present meeting, arrivals per meeting
+};
+
+__device__ __forceinline__ bool step_meet(StepMeet& meet) {
     __shared__ int ok;
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
-        *target += gridDim.x;
-        atomicAdd(ctr, 1u);
+        meet.target += meet.arrivals;
+        atomicAdd(meet.ctr, 1u);
         const long long t0 = clock64();
         bool in = true;
-        while ((int)(*(volatile unsigned*)ctr - *target) < 0) {
+        while ((int)(*(volatile unsigned*)meet.ctr - meet.target) < 0) {
             if (clock64() - t0 > kStepSpinCycles) { in = false; break; }
         }
         __threadfence();
@@ -416,7 +423,7 @@ __device__ __forceinline__ double step_total(const double* part) {
 template <int E>
 __device__ __forceinline__ bool step_gram_schmidt(const double* __restrict__ V, int m, int64_t n, int64_t e0, double* s_w,
                                                   double* s_c, double* rows, double* norm1, double* h0sq, double* h1sq,
-                                                  unsigned* ctr, unsigned* target) {
+                                                  StepMeet& meet) {
     constexpr int kPer = E / 32;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int G = gridDim.x;
@@ -452,7 +459,7 @@ __device__ __forceinline__ bool step_gram_schmidt(const double* __restrict__ V, 
         const double t = warp_sum8(acc, lane);
         if ((lane & 3) == 0 && j0 + (lane >> 2) <= m) rows[(int64_t)(j0 + (lane >> 2)) * G + blockIdx.x] = t;
     }
-    if (!step_meet(ctr, target)) return false;
+    if (!step_meet(meet)) return false;
     for (int j0 = wid * 8; j0 <= m; j0 += kStepThreads / 4) {
         double acc[8];
 #pragma unroll
@@ -505,7 +512,7 @@ __device__ __forceinline__ bool step_gram_schmidt(const double* __restrict__ V, 
         }
     }
     step_put(v, norm1);
-    if (!step_meet(ctr, target)) return false;
+    if (!step_meet(meet)) return false;
     *h1sq = step_total(norm1);
     return true;
 }
@@ -515,19 +522,21 @@ __device__ __forceinline__ bool step_gram_schmidt(const double* __restrict__ V, 
 // hold up the second one's product); sc[1]: beta for the next iteration;
 // beta_prev: beta of the iteration before (null at k = 0); part: scratch of
 // (5 + 2 m) gridDim.x doubles, m = k + 1; *ctr is a multiple of gridDim.x.
+// absent: arrivals that every meeting waits for beyond the grid's (0, but in
+// the test of the waits' limit).
 template <int E>
 __global__ void __launch_bounds__(kStepThreads) lanczos_step_kernel(double* __restrict__ V, int k,
                                                                     const double* __restrict__ w, int64_t n,
                                                                     double* sc, const double* beta_prev,
                                                                     double* part, unsigned* ctr, int always_twice,
-                                                                    double* host_sc) {
+                                                                    double* host_sc, int absent) {
     __shared__ double s_w[E];
     extern __shared__ double s_c[];   // k + 1 coefficients, |w|^2
     const int tid = threadIdx.x, G = gridDim.x, m = k + 1;
     const int64_t e0 = (int64_t)blockIdx.x * E;
     const double* vk = V + (int64_t)k * n;
-    unsigned target = 0;
-    if (tid == 0) target = *(volatile unsigned*)ctr / G * G;
+    StepMeet meet{ctr, 0u, (unsigned)(G + absent)};
+    if (tid == 0) meet.target = *(volatile unsigned*)ctr / G * G;
     double dot = 0.0;
     for (int q = tid; q < E; q += kStepThreads) {
         const int64_t e = e0 + q;
@@ -538,7 +547,7 @@ __global__ void __launch_bounds__(kStepThreads) lanczos_step_kernel(double* __re
     bool ok = true;
     double alpha = 0.0, h0sq = 0.0, h1sq = 0.0, bsq = 0.0;
     step_put(dot, part);
-    ok = step_meet(ctr, &target);
+    ok = step_meet(meet);
     if (ok) {
         alpha = step_total(part);
         const double b = beta_prev != nullptr ? beta_prev[0] : 0.0;
@@ -552,12 +561,12 @@ __global__ void __launch_bounds__(kStepThreads) lanczos_step_kernel(double* __re
         }
         __syncthreads();
         double* rows = part + 3 * (int64_t)G;
-        ok = step_gram_schmidt<E>(V, m, n, e0, s_w, s_c, rows, part + G, &h0sq, &h1sq, ctr, &target);
+        ok = step_gram_schmidt<E>(V, m, n, e0, s_w, s_c, rows, part + G, &h0sq, &h1sq, meet);
         bsq = h1sq;
         double again = 0.0;
         if (ok && (always_twice || h1sq < 0.5 * h0sq))
-            ok = step_gram_schmidt<E>(V, m, n, e0, s_w, s_c, rows + (int64_t)(m + 1) * G, part + 2 * G, &again, &bsq, ctr,
-                                      &target);
+            ok = step_gram_schmidt<E>(V, m, n, e0, s_w, s_c, rows + (int64_t)(m + 1) * G, part + 2 * G, &again, &bsq,
+                                      meet);
     }
     if (!ok) {
         if (tid == 0) host_sc[3] = 1.0;
@@ -642,13 +651,21 @@ cudaError_t lz_step(double* V, int k, const double* w, int64_t n, double* sc, co
     const int E = step_elems(n);
     const dim3 grid((unsigned)((n + E - 1) / E));
     const size_t dyn = (size_t)(k + 2) * sizeof(double);
-    void* args[] = {&V, &k, &w, &n, &sc, &beta_prev, &part, &ctr, &always_twice, &host_sc};
+    int absent = 0;
+#ifdef LM_DEBUG_BOUNDS
+    // tests of the host's side: a refused launch, a wait that runs out
+    const char* fault = std::getenv("LM_DEBUG_LANCZOS_STEP");
+    if (fault != nullptr && std::strcmp(fault, "refuse") == 0) return cudaErrorCooperativeLaunchTooLarge;
+    absent = fault != nullptr && std::strcmp(fault, "expire") == 0;
+#endif
+    void* args[] = {&V, &k, &w, &n, &sc, &beta_prev, &part, &ctr, &always_twice, &host_sc, &absent};
     const void* f = E == 64    ? (const void*)lanczos_step_kernel<64>
                     : E == 128 ? (const void*)lanczos_step_kernel<128>
                     : E == 256 ? (const void*)lanczos_step_kernel<256>
                                : (const void*)lanczos_step_kernel<512>;
-    count_launches(1);
-    return cudaLaunchCooperativeKernel(f, grid, dim3(kStepThreads), args, dyn, s);
+    const cudaError_t e = cudaLaunchCooperativeKernel(f, grid, dim3(kStepThreads), args, dyn, s);
+    if (e == cudaSuccess) count_launches(1);
+    return e;
 }
 
 cudaError_t lz_scale(const double* x, const double* nrm, double* y, int64_t n, cudaStream_t s) {

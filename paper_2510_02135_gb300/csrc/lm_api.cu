@@ -1098,10 +1098,17 @@ lm_status enqueue_lanczos_iteration(lm_solver* s, int k, int64_t n, double* V, d
         s->vprof_used += 1;
     }
     if (s->lz_one) {
-        LM_CUDA(lmk::lz_step(V, k, w, n, sk, k > 0 ? sk - kScal + 1 : nullptr, red,
-                             s->lzmeet.as<unsigned>(), s->reorth, s->pinned + kScal * k, s->stream),
-                "Lanczos iteration");
-    } else {
+        const cudaError_t e = lmk::lz_step(V, k, w, n, sk, k > 0 ? sk - kScal + 1 : nullptr, red,
+                                           s->lzmeet.as<unsigned>(), s->reorth, s->pinned + kScal * k, s->stream);
+        if (k == 0 && (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported)) {
+            // its CTAs do not fit the SMs this context may use: the separate kernels serve this call
+            cudaGetLastError();
+            s->lz_one = false;
+        } else {
+            LM_CUDA(e, "Lanczos iteration");
+        }
+    }
+    if (!s->lz_one) {
         LM_CUDA(lmk::lz_dot1(vk, w, n, red, ctr, sk, 0, s->stream), "alpha");
         // three-term update and |w| before the Gram-Schmidt pass
         LM_CUDA(lmk::lz_axpy2_norm(w, vk, sk, k > 0 ? vk - n : nullptr, k > 0 ? sk - kScal + 1 : nullptr, n, red, ctr,

@@ -282,7 +282,9 @@ cudaError_t lz_sub_vc_norm(const double* V, int m, const double* c, double* w, i
 // three-term update, Gram-Schmidt, beta (to sc[1]) and row k + 1 of V; the
 // scalars go to host_sc (page-locked, zeroed by the caller).  part: scratch of
 // lz_step_doubles(n, m_max) doubles (0: n or m_max out of its range, use the
-// separate kernels); *ctr: zero, or as the previous lz_step left it.
+// separate kernels); *ctr: zero, or as the previous lz_step left it.  Returns
+// cudaErrorCooperativeLaunchTooLarge, with nothing done, where the grid does
+// not fit the device.
 size_t lz_step_doubles(int64_t n, int m_max);
 cudaError_t lz_step(double* V, int k, const double* w, int64_t n, double* sc, const double* beta_prev, double* part,
                     unsigned* ctr, int always_twice, double* host_sc, cudaStream_t s);
