@@ -34,13 +34,23 @@ __device__ __forceinline__ double rsq(double x) { return 1.0 / sqrt(x); }
 // pair adds exactly nothing: four j are skipped together when that holds for
 // all of a warp's i.  At the roller example's b = 0.1 a that is r > 13 a,
 // nearly every pair.  A CTA takes kSoftBlock i-particles, and its four groups of
-// threads a quarter of every j-tile each.  N = 32768: 3.56 ms with one i per
-// thread and every pair evaluated.
+// threads a quarter of every j-tile each.  FP64 compares take the FP64 pipe,
+// which bounds that precision, so the tests for the range and for r = 0 read
+// the words of r^2 as integers there (the range by high words: pairs just
+// beyond it are evaluated and add zero).  N = 32768, one i per thread and every
+// pair evaluated / here: FP32 b = 0.1 a 3.56 / 0.81 ms, b = a 3.56 / 1.87; FP64
+// b = 0.1 a 109.8 / 106.7 ms, b = a 102.5 / 100.0 (107.5 with FP64 compares).
 template <typename R> constexpr R kExpZero = R(0);
 template <> constexpr float kExpZero<float> = 110.0f;     // -ln(2^-149) = 103.3
 template <> constexpr double kExpZero<double> = 760.0;    // -ln(2^-1074) = 744.4
 constexpr int kSoftBlock = 64;
 constexpr int kSoftGroups = 4;
+
+// Keys that order r^2 >= 0 as r^2 does (FP64: up to equal high words).
+__device__ __forceinline__ float range_key(float r2) { return r2; }
+__device__ __forceinline__ int range_key(double r2) { return __double2hiint(r2); }
+__device__ __forceinline__ bool apart(float r2) { return r2 > 0.0f; }
+__device__ __forceinline__ bool apart(double r2) { return __double_as_longlong(r2) != 0; }
 
 template <typename R>
 __global__ void __launch_bounds__(kSoftBlock* kSoftGroups)
@@ -56,7 +66,7 @@ __global__ void __launch_bounds__(kSoftBlock* kSoftGroups)
     const int64_t ii = live ? i : 0;
     const R xi = ld3<R>(pos, f64, 3 * ii), yi = ld3<R>(pos, f64, 3 * ii + 1), zi = ld3<R>(pos, f64, 3 * ii + 2);
     const R cut = d_pair + kExpZero<R> / inv_b;
-    const R cut2 = cut * cut * R(1.0001);   // above the rounding of r; infinite for an unbounded range
+    const auto cut2 = range_key(cut * cut * R(1.0001));   // above the rounding of r; infinite for an unbounded range
     R fx = R(0), fy = R(0), fz = R(0);
     for (int64_t jt = 0; jt < N; jt += NT) {
         const int64_t j = jt + threadIdx.x;
@@ -70,18 +80,18 @@ __global__ void __launch_bounds__(kSoftBlock* kSoftGroups)
         const int end = min(cnt, (grp + 1) * kSoftBlock);
         for (int jj = grp * kSoftBlock; jj < end; jj += 4) {
             R dx[4], dy[4], dz[4], r2[4];
-            R mn = R(0);
+            auto mn = cut2;
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const R4 p = sp[jj + u];
                 dx[u] = xi - p.x; dy[u] = yi - p.y; dz[u] = zi - p.z;
                 r2[u] = fma(dx[u], dx[u], fma(dy[u], dy[u], dz[u] * dz[u]));
-                mn = u == 0 ? r2[u] : fmin(mn, r2[u]);
+                mn = u == 0 ? range_key(r2[u]) : min(mn, range_key(r2[u]));
             }
             if (!__any_sync(0xffffffffu, mn <= cut2)) continue;
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                if (jj + u < end && r2[u] > R(0) && r2[u] <= cut2) {
+                if (jj + u < end && apart(r2[u]) && range_key(r2[u]) <= cut2) {
                     const R ir = rsq(r2[u]);
                     const R r = r2[u] * ir;
                     const R g = (r < d_pair) ? R(1) : expo((d_pair - r) * inv_b);
