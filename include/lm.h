@@ -301,7 +301,10 @@ lm_status lm_mdot_backward(lm_solver *solver, const void *forces, const void *to
  *   are bitwise reproducible too, and its partial sums take up to 128 slots of
  *   3 or 6 FP64 values per particle (or 256 MiB if that is more); when they do
  *   not fit, the one-sided kernel runs.  lm_set_pair_config pins the one-sided
- *   kernel for the solver; lm_autotune tunes it without pinning it.
+ *   kernel for the solver, even with the configuration that
+ *   lm_get_pair_config returns, which is the one-sided kernel's in every case;
+ *   giving the answer of lm_autotune back to the same solver at the same N
+ *   changes nothing.
  */
 /* Launch configuration of the pair kernels (no paper counterpart):
  *   threads: CTA size and j-tile length (128 or 256);
@@ -356,9 +359,13 @@ lm_status lm_set_adjoint_config(lm_solver *solver, const lm_pair_config *cfg);
  * keep the fastest, and return it in *best (nullable).  reps >= 1 timed
  * launches per candidate (after one warm-up launch); the three fastest are
  * then timed three more times each, interleaved, and the best of their four
- * timings decides.  For an LM_FP32C open solver without angular blocks it
- * also times the configurations of the adjoint kernel the same way and
- * keeps the fastest (lm_get_adjoint_config).  The choice is also recorded
+ * timings decides.  These are the configurations of the one-sided kernels.
+ * Where the library selects the symmetric one, that is timed too, and the
+ * winner takes its place only when it is faster by 2%; the solver uses the
+ * faster form from then on, and the answer need not be set.  For an LM_FP32C
+ * open solver without angular blocks it also times the configurations of the
+ * adjoint kernel the same way and keeps the fastest
+ * (lm_get_adjoint_config).  The choice is also recorded
  * for the process under (device, precision, angular flag, geometry,
  * floor(log2 N)): a solver without a configuration of its own (none set or
  * tuned) whose N falls in a recorded bucket starts from that choice, with

@@ -186,6 +186,8 @@ struct lm_solver {
     lm_pair_config cfg{128, 4, 1, 0};
     bool cfg_forced = false;
     bool cfg_pinned = false;   // set by lm_set_pair_config: that one-sided kernel, never the symmetric form
+    bool cfg_tuned = false;    // cfg is lm_autotune's choice on this solver
+    int one_sided_log2n = -1;  // N bucket in which the autotuner found cfg faster than the symmetric form
     int64_t cfg_N = -1;
     lmk::SymPlan sym{};        // symmetric form of the product, planned for sym_N particles
     bool sym_ok = false;
@@ -392,15 +394,20 @@ struct TunedEntry {
     lm_pair_config cfg;
     lm_pair_config adj;
     bool has_adj = false;
+    bool one_sided = false;   // cfg beat the symmetric form
     int64_t N = 0;
 };
 std::mutex g_tuned_mu;
 std::map<std::array<int, 5>, TunedEntry> g_tuned;
 
-std::array<int, 5> tuned_key(const lm_solver* s, int64_t N) {
+int log2_bucket(int64_t N) {
     int b = 0;
     while (b < 62 && ((int64_t)1 << (b + 1)) <= N) ++b;
-    return {s->device, s->fp64 ? 1 : 0, s->angular ? 1 : 0, s->wall ? 1 : 0, b};
+    return b;
+}
+
+std::array<int, 5> tuned_key(const lm_solver* s, int64_t N) {
+    return {s->device, s->fp64 ? 1 : 0, s->angular ? 1 : 0, s->wall ? 1 : 0, log2_bucket(N)};
 }
 
 // The process's record, else the persistent cache (LM_AUTOTUNE_CACHE).
@@ -418,7 +425,7 @@ bool lookup_tuned(const lm_solver* s, int64_t N, TunedEntry* e) {
     long long n = 0;
     bool has_adj = false;
     if (!lmk::tune_cache_key(s->device, key[1], key[2], key[3], key[4], &ck) ||
-        !lmk::tune_cache_lookup(ck, &n, &e->cfg, &e->adj, &has_adj))
+        !lmk::tune_cache_lookup(ck, &n, &e->cfg, &e->adj, &has_adj, &e->one_sided))
         return false;
     if (!pair_config_supported(s, e->cfg.threads, e->cfg.ilp, e->cfg.packed) || e->cfg.splits < 1) return false;
     e->N = n;
@@ -435,6 +442,7 @@ void ensure_config(lm_solver* s) {
     if (s->cfg_N == s->N) return;
     if (!s->cfg_forced) {
         s->cfg = default_config(s, s->N);
+        s->one_sided_log2n = -1;
         TunedEntry e;
         bool found = lookup_tuned(s, s->N, &e);
         if (!found && lmk::autotune_on_first_use()) {
@@ -445,6 +453,7 @@ void ensure_config(lm_solver* s) {
         }
         if (found) {
             s->cfg = e.cfg;
+            if (e.one_sided) s->one_sided_log2n = log2_bucket(s->N);
             if (e.N != s->N) {
                 const int occ = std::max(1, pair_ctas_per_sm(s, e.cfg.threads, e.cfg.ilp, e.cfg.packed));
                 s->cfg.splits = auto_splits(s->N, e.cfg.threads, e.cfg.ilp, occ * s->sm_count);
@@ -467,10 +476,12 @@ bool can_allocate(const lm_solver* s, const DBuf& partials, size_t bytes) {
 }
 
 // Whether the product takes the symmetric form: its rule selects this (precision,
-// blocks, geometry, N), no one-sided kernel is pinned and its partial sums fit
-// the device (else the one-sided form, which needs fewer, serves).
+// blocks, geometry, N), no one-sided kernel is pinned or was found faster by the
+// autotuner, and its partial sums fit the device (else the one-sided form,
+// which needs fewer, serves).
 bool sym_form(lm_solver* s) {
     if (s->cfg_pinned) return false;
+    if (s->one_sided_log2n >= 0 && s->one_sided_log2n == log2_bucket(s->N)) return false;
     if (s->sym_N != s->N) {
         s->sym_ok = lmk::sym_plan(s->fp64, s->angular, s->wall, s->N, s->sm_count, &s->sym);
         s->sym_N = s->N;
@@ -1439,7 +1450,12 @@ lm_status lm_set_pair_config(lm_solver* s, const lm_pair_config* cfg) {
     if (!pair_config_supported(s, cfg->threads, cfg->ilp, cfg->packed) || cfg->splits < 0)
         return fail(LM_ERR_INVALID_ARG, "unsupported pair configuration (threads %d, ilp %d, splits %d, packed %d)",
                     cfg->threads, cfg->ilp, cfg->splits, cfg->packed);
+    // the answer of this solver's own autotuning, given back: it is in use already, one-sided or symmetric
+    if (s->cfg_tuned && s->has_pos && s->cfg_N == s->N && cfg->threads == s->cfg.threads && cfg->ilp == s->cfg.ilp &&
+        cfg->splits == s->cfg.splits && cfg->packed == s->cfg.packed)
+        return LM_OK;
     s->cfg = *cfg;
+    s->cfg_tuned = false;
     if (s->cfg.splits == 0) {
         int occ = std::max(1, pair_ctas_per_sm(s, cfg->threads, cfg->ilp, cfg->packed));
         s->cfg.splits = s->has_pos ? auto_splits(s->N, cfg->threads, cfg->ilp, occ * s->sm_count) : 1;
@@ -1511,7 +1527,8 @@ lm_status autotune_impl(lm_solver* s, int reps, lm_pair_config* best) {
     // One timing of every candidate, then the three fastest again in three
     // interleaved rounds (the minimum of the four timings decides), so that
     // clock and scheduling noise of a single timing does not pick the winner.
-    auto pick = [&](auto&& launch, const std::vector<lm_pair_config>& cs, lm_pair_config* out) -> lm_status {
+    auto pick = [&](auto&& launch, const std::vector<lm_pair_config>& cs, lm_pair_config* out,
+                    float* best_ms = nullptr) -> lm_status {
         std::vector<std::pair<float, size_t>> t;
         for (size_t i = 0; i < cs.size(); ++i) {
             float ms = 0.f;
@@ -1532,13 +1549,36 @@ lm_status autotune_impl(lm_solver* s, int reps, lm_pair_config* best) {
         for (size_t q = 1; q < top; ++q)
             if (t[q].first < t[best_q].first) best_q = q;
         *out = cs[t[best_q].second];
+        if (best_ms) *best_ms = t[best_q].first;
         return LM_OK;
     };
     lm_pair_config best_cfg = default_config(s, N);
-    lm_status result = pick(
-        [&](const lm_pair_config& c) { return run_mdot(s, fin, fin + bytes, s->fp64, fout, fout + bytes, s->fp64, c,
-                                                    nullptr, true); },
-        cands, &best_cfg);
+    bool one_sided = true;
+    auto product = [&](const lm_pair_config& c) {
+        return run_mdot(s, fin, fin + bytes, s->fp64, fout, fout + bytes, s->fp64, c, nullptr, one_sided);
+    };
+    float one_ms = 0.f;
+    lm_status result = pick(product, cands, &best_cfg, &one_ms);
+    // The symmetric form, where the rule selects it: the one-sided winner takes
+    // its place only when it is faster by 2%, more than timings of one kernel
+    // differ (6N, N = 65536: 6.16 against 6.32 ms; at other sizes within 1.3%,
+    // with a fifth more error in the 256-thread configurations).
+    const int before = s->one_sided_log2n;
+    s->one_sided_log2n = -1;
+    if (result == LM_OK && sym_form(s)) {
+        one_sided = false;
+        float sym_ms = 0.f;
+        for (int round = 0; round < 4 && result == LM_OK; ++round) {
+            float ms = 0.f;
+            result = time_one(product, best_cfg, &ms);
+            sym_ms = round == 0 ? ms : std::min(sym_ms, ms);
+        }
+        one_sided = result == LM_OK && one_ms < 0.98f * sym_ms;
+        if (one_sided) s->one_sided_log2n = log2_bucket(N);
+    } else {
+        one_sided = false;   // no choice to record
+    }
+    if (result != LM_OK) s->one_sided_log2n = before;
     // the packed translation adjoint (open geometry): threads x ilp x j per vote x splits
     if (result == LM_OK && !s->fp64 && !s->angular && !s->wall) {
         std::vector<lm_pair_config> acands;
@@ -1574,10 +1614,12 @@ lm_status autotune_impl(lm_solver* s, int reps, lm_pair_config* best) {
     if (result != LM_OK) return result;
     s->cfg = best_cfg;
     s->cfg_forced = true;
+    s->cfg_tuned = true;
     s->cfg_N = N;
     {
         TunedEntry e;
         e.cfg = best_cfg;
+        e.one_sided = one_sided;
         e.N = N;
         e.has_adj = (s->adj_cfg_N == N) && !s->fp64 && !s->angular && !s->wall;
         if (e.has_adj) e.adj = s->adj_cfg;
@@ -1588,7 +1630,7 @@ lm_status autotune_impl(lm_solver* s, int reps, lm_pair_config* best) {
         }
         lmk::TuneCacheKey ck;
         if (lmk::tune_cache_key(s->device, key[1], key[2], key[3], key[4], &ck))
-            lmk::tune_cache_store(ck, N, best_cfg, e.has_adj ? &e.adj : nullptr);
+            lmk::tune_cache_store(ck, N, best_cfg, e.has_adj ? &e.adj : nullptr, one_sided);
     }
     if (best) *best = best_cfg;
     return LM_OK;

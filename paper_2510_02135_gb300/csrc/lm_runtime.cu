@@ -70,7 +70,7 @@ struct CacheEntry {
     TuneCacheKey key;
     long long n;
     lm_pair_config cfg, adj;
-    bool has_adj;
+    bool has_adj, one_sided;
 };
 
 bool g_cache_loaded = false;
@@ -106,6 +106,8 @@ void load_cache_locked() {
         e.has_adj = json_int(line, "adj_threads", &at) && json_int(line, "adj_ilp", &ail) &&
                     json_int(line, "adj_splits", &asp) && json_int(line, "adj_packed", &apk);
         if (e.has_adj) e.adj = lm_pair_config{(int)at, (int)ail, (int)asp, (int)apk};
+        long long one;
+        e.one_sided = json_int(line, "one_sided", &one) && one == 1;
         g_cache.push_back(e);   // a later line for the same key wins
     }
     std::fclose(f);
@@ -167,7 +169,7 @@ bool tune_cache_key(int device, int precision, int angular, int geometry, int lo
 }
 
 bool tune_cache_lookup(const TuneCacheKey& key, long long* n, lm_pair_config* cfg, lm_pair_config* adj,
-                       bool* has_adj) {
+                       bool* has_adj, bool* one_sided) {
     std::lock_guard<std::mutex> lk(g_rt_mu);
     load_cache_locked();
     for (size_t i = g_cache.size(); i-- > 0;) {
@@ -175,13 +177,15 @@ bool tune_cache_lookup(const TuneCacheKey& key, long long* n, lm_pair_config* cf
         *n = g_cache[i].n;
         *cfg = g_cache[i].cfg;
         *has_adj = g_cache[i].has_adj;
+        *one_sided = g_cache[i].one_sided;
         if (g_cache[i].has_adj) *adj = g_cache[i].adj;
         return true;
     }
     return false;
 }
 
-void tune_cache_store(const TuneCacheKey& key, long long n, const lm_pair_config& cfg, const lm_pair_config* adj) {
+void tune_cache_store(const TuneCacheKey& key, long long n, const lm_pair_config& cfg, const lm_pair_config* adj,
+                      bool one_sided) {
     std::lock_guard<std::mutex> lk(g_rt_mu);
     load_cache_locked();
     CacheEntry e{};
@@ -189,6 +193,7 @@ void tune_cache_store(const TuneCacheKey& key, long long n, const lm_pair_config
     e.n = n;
     e.cfg = cfg;
     e.has_adj = adj != nullptr;
+    e.one_sided = one_sided;
     if (adj) e.adj = *adj;
     g_cache.push_back(e);
     const char* path = env("LM_AUTOTUNE_CACHE");
@@ -203,6 +208,7 @@ void tune_cache_store(const TuneCacheKey& key, long long n, const lm_pair_config
     if (adj)
         std::fprintf(f, ",\"adj_threads\":%d,\"adj_ilp\":%d,\"adj_splits\":%d,\"adj_packed\":%d", adj->threads,
                      adj->ilp, adj->splits, adj->packed);
+    if (one_sided) std::fprintf(f, ",\"one_sided\":1");
     std::fprintf(f, "}\n");
     std::fclose(f);
 }

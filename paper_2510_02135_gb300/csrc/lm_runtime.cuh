@@ -35,8 +35,10 @@ struct TuneCacheKey {
 };
 bool tune_cache_key(int device, int precision, int angular, int geometry, int log2n, TuneCacheKey* key);
 bool tune_cache_lookup(const TuneCacheKey& key, long long* n, lm_pair_config* cfg, lm_pair_config* adj,
-                       bool* has_adj);
-void tune_cache_store(const TuneCacheKey& key, long long n, const lm_pair_config& cfg, const lm_pair_config* adj);
+                       bool* has_adj, bool* one_sided);
+// one_sided: cfg beat the symmetric product (where that form exists).
+void tune_cache_store(const TuneCacheKey& key, long long n, const lm_pair_config& cfg, const lm_pair_config* adj,
+                      bool one_sided);
 // LM_AUTOTUNE=1: a solver without a configuration of its own tunes the first
 // time it runs a product at an N bucket that no cache holds.
 int autotune_on_first_use();
