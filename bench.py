@@ -50,8 +50,7 @@ METRIC = "RPY pair-interactions/s (N^2 ordered pairs per application of M, incl.
 UNIT = "pair-interactions/s"
 FP32_LANES_PER_SM = 128
 RECIPE_MAX_SM_MHZ = 2070.0
-FLOPS_PER_PAIR_6N = 86
-FLOPS_PER_PAIR_TT = 35   # translation-only far-field pair (the batched and adjoint workloads)
+FLOPS_PER_PAIR_TT = 35   # translation-only far-field pair, one-sided (the batched workload)
 PAIR_KERNEL_SRCS = [os.path.join(ROOT, "paper_2510_02135_gb300", "csrc", f)
                     for f in ("pair_kernels.cu", "pair_common.cuh")]
 # ncu summaries of the forward pair kernel, per workload (DRAM bytes per launch)
@@ -169,6 +168,21 @@ def profile_traffic(workload: str):
         return float(vals["dram_bytes_per_launch"].split()[0])
     except (KeyError, ValueError, IndexError):
         return None
+
+
+def product_kernel(form, cfg, blocks: str, wall: bool = False) -> str:
+    """Name of the kernel that a solver's FP32 products run."""
+    if form["symmetric"]:
+        return (f"sym_mdot_x2_kernel (symmetric pair kernel, packed FP32, {blocks}; every unordered pair once, "
+                f"{form['flops_per_pair']:g} flops executed per ordered pair)")
+    name = ("rpy_wall" if wall else "rpy_mdot") + ("_x2_kernel" if cfg["packed"] else "_kernel")
+    return (f"{name} (one-sided pair kernel, {'packed' if cfg['packed'] else 'scalar'} FP32, {blocks}, "
+            f"{form['flops_per_pair']:g} flops per ordered pair)")
+
+
+def executed_tflops(form, pairs: float, ms: float) -> float:
+    """Rate of the flops that the product's kernel spends on `pairs` ordered pairs."""
+    return form["flops_per_pair"] * pairs / (ms / 1e3) / 1e12
 
 
 def fp32_peak(local: int):
@@ -324,14 +338,13 @@ def hotpath_leg(workload, steps, warmup, dist, local, *, pair_config=None, autot
                "api": "lm_set_positions/lm_mdot/lm_sqrt_mdot with pinned host buffers"}
 
     peak, sms = fp32_peak(local)
-    achieved = prof["pair_flops"] / (prof["pair_ms"] / 1e3) / 1e12 if prof["pair_ms"] > 0 else None
+    form = lm.lm_get_product_form(solver)
+    achieved = executed_tflops(form, prof["pair_interactions"], prof["pair_ms"]) if prof["pair_ms"] > 0 else None
     roofline = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-                "frac": (achieved / peak) if achieved else None, "traffic": profile_traffic(workload),
-                "kernel": ("sym_mdot_x2_kernel (symmetric pair kernel, packed FP32, all four blocks; every unordered "
-                           "pair once, flops counted per ordered pair)" if n < 100_000 and not pair_config
-                           else "rpy_mdot_x2_kernel (forward pair kernel, packed FP32, all four blocks)" if cfg["packed"]
-                           else "rpy_mdot_kernel (forward pair kernel, scalar FP32, all four blocks)"),
-                "flops_per_pair": FLOPS_PER_PAIR_6N, "pairs_per_launch": float(n) * n,
+                "frac": (achieved / peak) if achieved else None,
+                "traffic": None if form["symmetric"] else profile_traffic(workload),
+                "kernel": product_kernel(form, cfg, "all four blocks"),
+                "flops_per_pair": form["flops_per_pair"], "pairs_per_launch": float(n) * n,
                 "pair_launches": prof["pair_launches"],
                 "pair_kernel_ms_avg": prof["pair_ms"] / max(1, prof["pair_launches"]),
                 "pair_share_of_step": prof["pair_ms"] / max(1e-9, total_ms),
@@ -388,7 +401,8 @@ def hotpath_leg(workload, steps, warmup, dist, local, *, pair_config=None, autot
                           "(k+1) n FMAs) each at max(HBM time, FMA time at the measured FP64 rate); the DGKS second "
                           "pass, rarely taken, not counted"})
     return {"workload": workload, "desc": desc, "n": n, "value": value, "ms_per_step": total_ms_max / steps,
-            "steps": steps, "warmup": warmup, "iters": list(iters), "cfg": cfg, "autotune_s": t_tune,
+            "steps": steps, "warmup": warmup, "iters": list(iters),
+            "cfg": None if form["symmetric"] else cfg, "autotune_s": t_tune,
             "roofline": roofline, "lanczos_vectors": lanczos_vectors, "e2e": e2e, "launches": launches,
             "clocks": clocks, "wall_s_timed": t_wall, "lanczos_stats": stats, "tol": tol,
             "_solver": solver, "_s": s_, "_eta": eta, "_a": a, "_lin": lin, "_ang": ang, "_F": F, "_T": T}
@@ -513,7 +527,8 @@ def adjoint_leg(steps, warmup, dist, local, *, pair_config=None, adjoint_config=
     peak, _ = fp32_peak(local)
     fwd_ms = float(np.median(fwd))
     bwd_ms = float(np.median(bwd))
-    achieved = FLOPS_PER_PAIR_TT * float(n) * n / (fwd_ms / 1e3) / 1e12
+    form, cfg = lm.lm_get_product_form(solver), lm.lm_get_pair_config(solver)
+    achieved = executed_tflops(form, float(n) * n, fwd_ms)
 
     # the same suspension with angular blocks (torques T, cotangents H): the
     # forward product M [F; T] and the adjoint (dX, dF, dT) in their default
@@ -541,7 +556,8 @@ def adjoint_leg(steps, warmup, dist, local, *, pair_config=None, adjoint_config=
     fwd6 = float(np.median([e[0].elapsed_time(e[1]) for e in ev6]))
     bwd6 = float(np.median([e[1].elapsed_time(e[2]) for e in ev6]))
     angular = {"forward_ms": fwd6, "backward_ms": bwd6, "backward_over_forward": bwd6 / fwd6,
-               "steps": 3, "pair_config": lm.lm_get_pair_config(solver6),
+               "steps": 3,
+               "pair_config": None if lm.lm_get_product_form(solver6)["symmetric"] else lm.lm_get_pair_config(solver6),
                "adjoint_config": lm.lm_get_adjoint_config(solver6),
                "desc": "same N and positions with torques; backward = dX, dF, dT (the default symmetric form)"}
     del solver6
@@ -551,10 +567,10 @@ def adjoint_leg(steps, warmup, dist, local, *, pair_config=None, adjoint_config=
                     f"step = lm_mdot + lm_mdot_backward (dX, dF)",
             "forward_ms": fwd_ms, "backward_ms": bwd_ms, "backward_over_forward": bwd_ms / fwd_ms,
             "target_backward_over_forward": 2.5,
-            "pair_config": lm.lm_get_pair_config(solver), "adjoint_config": lm.lm_get_adjoint_config(solver),
+            "pair_config": None if form["symmetric"] else cfg, "adjoint_config": lm.lm_get_adjoint_config(solver),
             "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                          "frac": achieved / peak, "traffic": None,
-                         "kernel": "forward pair kernel (translation, 35 flops/pair)"},
+                         "kernel": product_kernel(form, cfg, "translation")},
             "gpu_launches": launches, "clocks": clocks, "angular": angular,
             "l2": "flushed by a 256 MB device write before every step"}
 
@@ -858,13 +874,6 @@ def run_single(args, ws, rank, local, pcfg, acfg):
     return 0
 
 
-# Algorithmic flops of one ordered pair above a single wall, translation
-# blocks (FMA = 2, counted from the formulas as the kernel evaluates them):
-# the free-space far-field pair (35) plus the wall part (96); the library's
-# profile counters use the same figure.
-WALL_FLOPS_PER_PAIR_TT = 131
-
-
 def run_wall(args, ws, rank, local, dist):
     """Mobility product above a single no-slip wall (the paper's "bottom
     wall" benchmark shape): N = 32768 spheres uniform in a cube on the wall at
@@ -924,20 +933,19 @@ def run_wall(args, ws, rank, local, dist):
     props = torch.cuda.get_device_properties(local)
     peak = props.multi_processor_count * FP32_LANES_PER_SM * 2 * RECIPE_MAX_SM_MHZ * 1e6 / 1e12
     kern_ms = prof["pair_ms"] / max(1, prof["pair_launches"])
-    achieved = prof["pair_flops"] / (prof["pair_ms"] / 1e3) / 1e12
+    form, cfg = lm.lm_get_product_form(solver), lm.lm_get_pair_config(solver)
+    achieved = executed_tflops(form, prof["pair_interactions"], prof["pair_ms"])
     line = {"metric": METRIC, "value": pairs / (tmax / 1e3), "unit": UNIT, "n_gpus": ws, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": tmax / args.steps, "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None, "dtype": "f32", "data": "synthetic (seeded)",
             "config": {"workload": f"wall_n32768: N={n} spheres uniform in a cube resting on a no-slip wall, "
                                    f"number density {c['rho']}/a^3, forces only, FP32 compensated; "
                                    f"step = lm_set_positions + lm_mdot",
-                       "pair_config": lm.lm_get_pair_config(solver),
+                       "pair_config": None if form["symmetric"] else cfg,
                        "l2": "flushed by a 256 MB device write before every step"},
             "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                          "frac": achieved / peak, "traffic": None,
-                         "kernel": "single-wall pair kernel (%s, translation, %d flops/pair)"
-                                   % ("packed" if lm.lm_get_pair_config(solver)["packed"] else "scalar",
-                                      WALL_FLOPS_PER_PAIR_TT),
+                         "kernel": product_kernel(form, cfg, "single wall, translation", wall=True),
                          "pair_kernel_ms_avg": kern_ms},
             "gpu_launches": launches, "clocks": clocks}
     if rank == 0:
@@ -1023,7 +1031,8 @@ def run_rollers(args, ws, rank, local, dist):
                                    f"(product, RFD drift, Lanczos tol {c['tol']}), FP32 pairs, all blocks",
                        "lanczos_iterations_mean": float(np.mean(iters)),
                        "preconditioner": "jacobi" if args.jacobi else "none",
-                       "pair_config": lm.lm_get_pair_config(solver),
+                       "pair_config": None if lm.lm_get_product_form(solver)["symmetric"]
+                       else lm.lm_get_pair_config(solver),
                        "l2": "flushed by a 256 MB device write before every step (outside the step events)"},
             "gpu_launches": launches, "clocks": clocks}
     if rank == 0:

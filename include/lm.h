@@ -328,6 +328,13 @@ typedef struct {
 lm_status lm_get_pair_config(lm_solver *solver, lm_pair_config *cfg);
 lm_status lm_set_pair_config(lm_solver *solver, const lm_pair_config *cfg);
 
+/* lm_get_product_form -- which kernel the products of the solver's current N
+ * run: *symmetric is 1 for the symmetric one, 0 for the one-sided one, and
+ * *flops_per_pair (nullable) the flops that it spends per ordered pair: 35
+ * (forces only), 86 (all blocks), 131 and 299 (single wall) one-sided; 25.5,
+ * 72, 85 and 222 symmetric.  Positions must be set. */
+lm_status lm_get_product_form(lm_solver *solver, int *symmetric, double *flops_per_pair);
+
 /* lm_get_adjoint_config / lm_set_adjoint_config -- launch configuration of
  * lm_mdot_backward for the current N.  LM_FP32C without angular blocks (the
  * packed kernels): threads 128 or 256, ilp 2 or 4, and packed
@@ -407,7 +414,8 @@ typedef struct {
     double pair_ms;           /* their summed device time, milliseconds */
     double pair_interactions; /* ordered pairs evaluated, N^2 per launch */
     double pair_flops;        /* algorithmic flops: 35 per pair (forces only) or 86 (all blocks);
-                                 single wall: 131 or 299 */
+                                 single wall: 131 or 299; whichever kernel ran (see
+                                 lm_get_product_form for what it spends) */
     int64_t vector_iterations; /* Lanczos iterations whose vector kernels were timed */
     double vector_ms;          /* their summed device time, milliseconds */
     double vector_bytes;       /* their algorithmic bytes (see above) */

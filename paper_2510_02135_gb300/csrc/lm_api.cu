@@ -1444,6 +1444,19 @@ lm_status lm_get_pair_config(lm_solver* s, lm_pair_config* cfg) {
     return LM_OK;
 }
 
+lm_status lm_get_product_form(lm_solver* s, int* symmetric, double* flops_per_pair) {
+    if (lm_status st = check_solver(s, true)) return st;
+    if (symmetric == nullptr) return fail(LM_ERR_INVALID_ARG, "symmetric is NULL");
+    DeviceGuard g(s->device);
+    ensure_config(s);
+    *symmetric = sym_form(s) ? 1 : 0;
+    if (flops_per_pair)
+        *flops_per_pair = !*symmetric ? solver_flops_per_pair(s)
+                          : s->wall   ? (s->angular ? lmk::kFlopsPerPairSymWall6N : lmk::kFlopsPerPairSymWallTT)
+                                      : (s->angular ? lmk::kFlopsPerPairSym6N : lmk::kFlopsPerPairSymTT);
+    return LM_OK;
+}
+
 lm_status lm_set_pair_config(lm_solver* s, const lm_pair_config* cfg) {
     if (lm_status st = check_solver(s, false)) return st;
     if (cfg == nullptr) return fail(LM_ERR_INVALID_ARG, "cfg is NULL");

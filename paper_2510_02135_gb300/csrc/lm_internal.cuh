@@ -87,6 +87,13 @@ constexpr double kFlopsPerPair6N = 86.0;
 // the formulas as wall_kernels.cu evaluates them.
 constexpr double kFlopsPerPairWallTT = 131.0;
 constexpr double kFlopsPerPairWall6N = 299.0;
+// What the symmetric kernels spend per ordered pair (half of an unordered
+// one's; counted from sym_far2 and sym_wall2, FMA = 2, reciprocal square roots
+// not counted): coefficients once, the application for both particles.
+constexpr double kFlopsPerPairSymTT = 25.5;
+constexpr double kFlopsPerPairSym6N = 72.0;
+constexpr double kFlopsPerPairSymWallTT = 85.0;
+constexpr double kFlopsPerPairSymWall6N = 222.0;
 
 // Constants of the RPY pair blocks for radius a, in units of 1/(8 pi eta).
 // Far field (r >= 2a), d = x_i - x_j, F the force and T the torque on j:

@@ -113,6 +113,8 @@ def lib():
         L.lm_mdot_backward.restype = st
         L.lm_get_pair_config.argtypes = [_vp, ctypes.POINTER(lm_pair_config)]
         L.lm_get_pair_config.restype = st
+        L.lm_get_product_form.argtypes = [_vp, ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_double)]
+        L.lm_get_product_form.restype = st
         L.lm_set_pair_config.argtypes = [_vp, ctypes.POINTER(lm_pair_config)]
         L.lm_set_pair_config.restype = st
         L.lm_get_adjoint_config.argtypes = [_vp, ctypes.POINTER(lm_pair_config)]
@@ -604,6 +606,13 @@ def lm_get_pair_config(s: Solver) -> dict:
     c = lm_pair_config()
     _check(lib().lm_get_pair_config(s.handle, ctypes.byref(c)))
     return {"threads": c.threads, "ilp": c.ilp, "splits": c.splits, "packed": c.packed}
+
+
+def lm_get_product_form(s: Solver) -> dict:
+    """Which kernel the solver's products run, and its flops per ordered pair."""
+    y, f = ctypes.c_int(0), ctypes.c_double(0.0)
+    _check(lib().lm_get_product_form(s.handle, ctypes.byref(y), ctypes.byref(f)))
+    return {"symmetric": bool(y.value), "flops_per_pair": f.value}
 
 
 def lm_set_pair_config(s: Solver, threads: int, ilp: int, splits: int = 0, packed: int = 0) -> None:
