@@ -448,7 +448,7 @@ __device__ __forceinline__ bool step_gram_schmidt(const double* __restrict__ V, 
                 const int64_t e = e0 + (q + h) * 32 + lane;
                 const int64_t ec = e < n ? e : n - 1;
 #pragma unroll
-                for (int r = 0; r < 8; ++r) x[h][r] = row[r][ec];
+                for (int r = 0; r < 8; ++r) x[h][r] = LM_INBOUNDS(ec >= 0, 16, ec) ? row[r][ec] : 0.0;
             }
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
@@ -457,7 +457,8 @@ __device__ __forceinline__ bool step_gram_schmidt(const double* __restrict__ V, 
             }
         }
         const double t = warp_sum8(acc, lane);
-        if ((lane & 3) == 0 && j0 + (lane >> 2) <= m) rows[(int64_t)(j0 + (lane >> 2)) * G + blockIdx.x] = t;
+        if ((lane & 3) == 0 && j0 + (lane >> 2) <= m && LM_INBOUNDS(G <= 152, 17, G))
+            rows[(int64_t)(j0 + (lane >> 2)) * G + blockIdx.x] = t;
     }
     if (!step_meet(meet)) return false;
     for (int j0 = wid * 8; j0 <= m; j0 += kStepThreads / 4) {
