@@ -342,14 +342,15 @@ lm_status lm_get_product_form(lm_solver *solver, int *symmetric, double *flops_p
  *     j-range chunks per i-block;
  *   3: the symmetric kernel: each unordered pair is evaluated once and added
  *     to both particles (the gradient of a pair term is odd in x_i - x_j and
- *     the tt block even), a quarter less time at N = 65536; splits = least
+ *     the tt block even), a quarter less time at N = 65536; the default
+ *     from N = 3000 on (ilp 4 above N = 10000); splits = least
  *     tiles (of `threads` particles) per work item, 0: chosen from N;
  * otherwise (LM_FP64, or angular blocks) threads 128 and packed
  *   3: the symmetric scalar kernel (the LM_FP64 default): each unordered
  *     pair once, its gradient added to one particle and subtracted from the
  *     other, the mobility parts of both directions from the same
- *     coefficients; ilp 1 (LM_FP64) or 2, 4 (LM_FP32C); 1.5x faster than
- *     packed 0 at N = 16384 (FP64, angular);
+ *     coefficients; ilp 1 (LM_FP64) or 2, 4 (LM_FP32C); 1.7x faster than
+ *     packed 0 at N = 8001 (FP64, angular);
  *   4: the same in packed f32x2 form, two i-particles per instruction
  *     (LM_FP32C with angular blocks, ilp 2 or 4; the default there, ilp 4
  *     above N = 10000): 1.7x faster than packed 0 at N = 65536;

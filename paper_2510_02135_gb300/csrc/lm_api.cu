@@ -359,8 +359,8 @@ lm_pair_config default_config(const lm_solver* s, int64_t N) {
     c.ilp = s->fp64 ? (s->angular ? 1 : 2) : (s->angular ? 4 : 8);
     c.packed = s->fp64 ? 0 : 1;
     if (!s->fp64 && s->angular && !s->wall && N >= 100000) {
-        // many i-blocks: eight i-particles per thread and four j per vote (131072: 25.4 / 25.7 ms, 524288: 403 / 412
-        // with rsqrtf; 23.8 and 376 since)
+        // many i-blocks: eight i-particles per thread and four j per vote (256 x 4 with one j per vote / this, ms:
+        // 99000 14.77 / 14.15, 131072 24.10 / 23.82, 262144 96.2 / 94.7)
         c.ilp = 8;
         c.packed = 4;
     }
@@ -582,14 +582,15 @@ lm_pair_config one_sided_adjoint_config(const lm_solver* s) {
 }
 
 // Adjoint launch configuration (item sizes chosen at launch): the symmetric
-// kernels, except for small FP32 translation-only systems.  Time per call,
-// ilp 2 / 4 / one-sided: FP32 translation N = 2048 41 / - / 37 us, 3000 55 / 60
-// / 96, 4096 55 / 64 / 95, 8192 132 / 144 / 203, 16384 450 / 427 / 606, 65536
-// 6.61 / 6.27 / 8.43 ms; with angular blocks 1024 64 / 103 / 177 us, 4096 103 /
-// 109 / 174, 16384 1156 / 1061 / 1776, 65536 17.1 / 15.5 / 27.0 ms.  FP64 (ilp
-// 1): 1024 0.12 / 1.17 ms, 8001 4.97 / 8.48 ms; with angular blocks 4096 3.18 /
-// 5.91 ms.  (With rsqrtf; the symmetric ones since: 4096 48 us, 8192 123, 65536
-// 5.88 ms; with angular blocks 1024 60 us, 4096 95, 16384 1022, 65536 15.3 ms.)
+// kernels, except for small FP32 translation-only systems.  Device time, us,
+// ilp 2 / 4 | one-sided: FP32 translation N = 1000 31 / 48 | 28, 2048 32 / 48 |
+// 29, 3000 42 / 48 | 37, 3100 43 / 48 | 45, 4096 44 / 48 | 56, 8192 118 / 127 |
+// 172, 16384 424 / 399 | 615, 65536 6397 / 5873 | 8077 (the one-sided form is
+// overtaken where its tiles of 128 pass 24, N = 3072); with angular blocks 1024
+// 55 / 94 | 168, 4096 89 / 95 | 171, 10000 442 / 445 | 766, 16384 1094 / 1015 |
+// 1754, 65536 16497 / 15215 | 26728.  FP64 (ilp 1): 1024 105 | 1171, 4096 1314 |
+// 2281, 8001 4923 | 8465; with angular blocks 1024 245 | 3007, 4096 3153 | 5924,
+// 8001 12030 | 20567.
 lm_pair_config default_adjoint_config(const lm_solver* s) {
     if (s->fp64) return lm_pair_config{128, 1, 0, 3};
     const int ilp = s->N <= 10000 ? 2 : 4;
@@ -1207,8 +1208,8 @@ static lm_status sqrt_mdot_body(lm_solver* s, const double* W, uint64_t seed, do
     }
     if (s->lz_one) {
         // the one-launch iteration's meeting counter (another n: another grid)
-        // and the host's scalars, among them its error words, start at zero;
-        // an earlier call may have left an iteration running ahead
+        // and the host's scalars, among them its error words, start at zero
+        // (an earlier call has waited for the iteration that ran ahead)
         LM_CUDA(s->lzmeet.ensure(64), "allocating counters");
         LM_CUDA(cudaMemsetAsync(s->lzmeet.p, 0, 64, s->stream), "allocating counters");
     }

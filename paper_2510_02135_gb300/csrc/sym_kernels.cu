@@ -702,11 +702,13 @@ cudaError_t sym_form(int fp64, int angular, int wall, const SymPlan& p, const Md
 
 // Products that take the symmetric form.  FP64 with a wall does not (its
 // one-sided kernel has no packed form to share the wall part with), nor FP32
-// with all blocks in free space from N = 100000 on: 46 against 41.5 operations
-// pay for the j-side up to there (65536: 6.49 / 6.61 ms), but no longer when
-// the one-sided kernel runs eight i-particles and four j per vote (131072: 25.4
-// / 25.4 ms, 262144: 101.1 / 101.2 ms; 65536 since the far field takes the bare
-// reciprocal root: 6.31 / 6.20 ms, 50000 3.69 / 3.97, 99000 14.2 / 15.6).
+// with all blocks in free space from N = 100000 on: 41.5 against 46 operations
+// do not pay for the j-side once the one-sided kernel has enough i-blocks for
+// eight i-particles per thread and four j per vote (256 x 8).  Device time,
+// symmetric / 256 x 8, ms: 40000 2.49 / 2.50, 50000 3.70 / 3.69, 65536 6.32 /
+// 6.28, 80000 9.37 / 9.30, 99000 14.23 / 14.15, 131072 24.76 / 23.81, 262144
+// 98.6 / 94.6, 524288 394 / 379.  Below the line they are within 1%, and the
+// symmetric sums are closer to FP64 (N = 65536: 4.2e-7 / 5.1e-7 of u).
 static bool sym_selected(int fp64, int angular, int wall, int64_t N) {
     return wall ? !fp64 : (fp64 || !angular || N < 100000);
 }
@@ -714,25 +716,28 @@ static bool sym_selected(int fp64, int angular, int wall, int64_t N) {
 // i-particles per thread and particles per j-tile.  Small systems are bound by
 // the latency of one item, so short tiles and few i-particles make more and
 // shorter items; large ones by the FMA pipe, where more i-particles share a
-// j-value and its shuffles.  Device time of a product on GB300, us (taken with
-// rsqrtf; the bare instruction took 4-7% off either side since: 50021 1422,
-// 32768 all blocks 1628, wall 1780, wall with all blocks 4610), symmetric at
+// j-value and its shuffles.  Device time of a product on GB300, us, symmetric at
 // (2, 32) / (2, 64) / (4, 128) / (8, 128) and one-sided with its default:
-//   forces, free space   N = 100   11 /  15 /  28 /    - |   22
-//                           1000   13 /  16 /  31 /    - |   24
-//                           4096   26 /  24 /  31 /    - |   33
-//                           8192   68 /  62 /  64 /    - |   84
-//                          16384  250 / 215 / 191 /  205 |  281
-//                          50021    - /   - /1570 / 1523 | 2164
-//   all blocks, free space  1000   15 /  22 |  27     4096  47 / 46 | 51     10000  - / 198 / 207 / 209 | 225
-//                          16384    - / 497 / 458 / 474 | 495     32768  - / 1811 / 1715 / 1674 | 1734
-//   forces, wall            1000   16 /  23 /  60 |  36   4096  49 /  48 /  56 | 73
-//                          16384  518 / 518 / 498 | 779
-//   all blocks, wall, (2, 32) / (2, 128)   1000   23 / 66 | 51   4096   99 / 105 | 130
-//                          32768  4800 / 4724 | 5970
-//   FP64 at 8 / 16 / 32 (the FP64 pipe is full at one warp per SM quarter): forces 200: 18 / 29 / 52 |
-//   185, 1024: 50 / 47 / 52 | 179, 8001: 2143 / 2115 / 2100 | 4334; all blocks 200: 32 / 56 / 105 |
-//   330, 1024: 112 / 101 / 104 | 318, 8001: 4863 / 4814 / 4791 | 8167
+//   forces, free space   N = 100   11 /  13 /  26 /   35 |   21
+//                           1000   12 /  15 /  28 /   39 |   22
+//                           4096   25 /  23 /  28 /   41 |   32
+//                           8192   72 /  61 /  60 /   63 |   78
+//                          16384  244 / 206 / 179 /  193 |  255
+//                          32768  751 / 720 / 650 /  640 |  845
+//                          50021 1686 /1627 /1445 / 1421 | 1916
+//   all blocks, free space  1000   14 /  21 /  50 /   59 |   26
+//                           4096   51 /  47 /  51 /   82 |   49
+//                          10000  217 / 193 / 201 /  201 |  216
+//                          16384  482 / 485 / 445 /  454 |  473
+//                          32768 1805 /1767 /1667 / 1629 | 1627
+//                          65536 7323 /7147 /6643 / 6303 | 6197
+//   forces, wall            1000   15 /  21 /  49 |   31     4096   46 /   46 /   49 |   67
+//                          16384  495 / 493 / 470 |  719    32768 1882 / 1871 / 1775 | 2600
+//   all blocks, wall, (2, 32) / (2, 128)   1000   21 /   59 |   45    4096   99 /  100 |  124
+//                                         16384 1203 / 1181 | 1615   32768 4686 / 4604 | 5700
+//   FP64 at 8 / 16 / 32 (the FP64 pipe is full at one warp per SM quarter):
+//   forces      200   18 /   29 /   52 |  160    1024   50 /   48 /   52 |  151    8001 2138 / 2113 / 2100 | 3390
+//   all blocks  200   32 /   56 /  105 |  306    1024  110 /  100 /  105 |  290    8001 4861 / 4811 / 4793 | 7168
 static void sym_tiling(int fp64, int angular, int wall, int64_t N, int* ilp, int* tile) {
     *ilp = fp64 ? 1 : 2;
     *tile = !fp64 || N > 3000 ? 32 : (N <= 800 ? 8 : 16);
