@@ -51,16 +51,16 @@ UNIT = "pair-interactions/s"
 FP32_LANES_PER_SM = 128
 RECIPE_MAX_SM_MHZ = 2070.0
 FLOPS_PER_PAIR_TT = 35   # translation-only far-field pair, one-sided (the batched workload)
-PAIR_KERNEL_SRCS = [os.path.join(ROOT, "paper_2510_02135_gb300", "csrc", f)
-                    for f in ("pair_kernels.cu", "pair_common.cuh")]
-# ncu summaries of the forward pair kernel, per workload (DRAM bytes per launch)
-PAIR_PROFILE = {"melt": "pair_kernel_melt_n524288.txt", "rpy6": "pair_kernel_rpy6_n32768.txt"}
+# ncu summaries of the product's kernel (DRAM bytes per launch), per workload and form (symmetric or one-sided)
+PAIR_PROFILE = {("melt", False): "pair_kernel_melt_n524288.txt", ("rpy6", True): "sym_kernel_rpy6_n32768.txt"}
+PAIR_KERNEL_SRCS = {False: ("pair_kernels.cu", "pair_common.cuh"),
+                    True: ("sym_kernels.cu", "sym_common.cuh", "pair_common.cuh")}
 
 
-def pair_kernel_source_hash() -> str:
+def pair_kernel_source_hash(symmetric: bool) -> str:
     h = hashlib.sha256()
-    for f in PAIR_KERNEL_SRCS:
-        h.update(open(f, "rb").read())
+    for f in PAIR_KERNEL_SRCS[symmetric]:
+        h.update(open(os.path.join(ROOT, "paper_2510_02135_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:16]
 
 
@@ -148,10 +148,11 @@ def measured_hbm_gbs():
         return 6800.0
 
 
-def profile_traffic(workload: str):
-    """DRAM bytes per pair-kernel launch from the committed ncu summary of this
-    workload, if it was taken on the current kernel source (else None)."""
-    name = PAIR_PROFILE.get(workload)
+def profile_traffic(workload: str, symmetric: bool):
+    """DRAM bytes per launch of the product's kernel from the committed ncu
+    summary of this workload and form, if it was taken on the current kernel
+    source (else None)."""
+    name = PAIR_PROFILE.get((workload, symmetric))
     if name is None:
         return None
     path = os.path.join(ROOT, "profiles", name)
@@ -162,7 +163,7 @@ def profile_traffic(workload: str):
         if ":" in line:
             k, v = line.split(":", 1)
             vals[k.strip()] = v.strip()
-    if (vals.get("kernel_source_sha256_16", "").split() or [""])[0] != pair_kernel_source_hash():
+    if (vals.get("kernel_source_sha256_16", "").split() or [""])[0] != pair_kernel_source_hash(symmetric):
         return None
     try:
         return float(vals["dram_bytes_per_launch"].split()[0])
@@ -342,7 +343,7 @@ def hotpath_leg(workload, steps, warmup, dist, local, *, pair_config=None, autot
     achieved = executed_tflops(form, prof["pair_interactions"], prof["pair_ms"]) if prof["pair_ms"] > 0 else None
     roofline = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": (achieved / peak) if achieved else None,
-                "traffic": None if form["symmetric"] else profile_traffic(workload),
+                "traffic": profile_traffic(workload, form["symmetric"]),
                 "kernel": product_kernel(form, cfg, "all four blocks"),
                 "flops_per_pair": form["flops_per_pair"], "pairs_per_launch": float(n) * n,
                 "pair_launches": prof["pair_launches"],
@@ -822,7 +823,6 @@ def main():
             step2_sum["error"] = err2
         else:
             step2_sum = _leg_summary(step2)
-        step2_sum["roofline"]["traffic"] = profile_traffic("rpy6")
         line["rpy6_n32768"] = step2_sum
         del step2
         torch.cuda.empty_cache()
