@@ -654,9 +654,10 @@ cudaError_t lz_step(double* V, int k, const double* w, int64_t n, double* sc, co
     const size_t dyn = (size_t)(k + 2) * sizeof(double);
     int absent = 0;
 #ifdef LM_DEBUG_BOUNDS
-    // tests of the host's side: a refused launch, a wait that runs out
+    // tests of the host's side: a refused launch (of every iteration, or from the third on), a wait that runs out
     const char* fault = std::getenv("LM_DEBUG_LANCZOS_STEP");
-    if (fault != nullptr && std::strcmp(fault, "refuse") == 0) return cudaErrorCooperativeLaunchTooLarge;
+    if (fault != nullptr && (std::strcmp(fault, "refuse") == 0 || (k >= 2 && std::strcmp(fault, "refuse_later") == 0)))
+        return cudaErrorCooperativeLaunchTooLarge;
     absent = fault != nullptr && std::strcmp(fault, "expire") == 0;
 #endif
     void* args[] = {&V, &k, &w, &n, &sc, &beta_prev, &part, &ctr, &always_twice, &host_sc, &absent};

@@ -1166,6 +1166,13 @@ void settle_vector_profile(lm_solver* s, int64_t n) {
 
 }  // namespace
 
+// Waits for the stream when it goes out of scope: iterations in flight write the
+// solver's page-locked scalars and basis, which a later call may replace.
+struct StreamWait {
+    cudaStream_t stream;
+    ~StreamWait() { cudaStreamSynchronize(stream); }
+};
+
 static lm_status sqrt_mdot_body(lm_solver* s, const double* W, uint64_t seed, double prefactor, double tol, int max_iter,
                        void* lin_out, void* ang_out, int* iters_out) {
     if (lm_status st = check_solver(s, true)) return st;
@@ -1250,6 +1257,7 @@ static lm_status sqrt_mdot_body(lm_solver* s, const double* W, uint64_t seed, do
     LM_CUDA(lmk::lz_scale(dW, wn, V, n, s->stream), "normalise W");
     LM_CUDA(cudaMemcpyAsync(s->pinned + kScal * (m_max + 2), wn, sizeof(double), cudaMemcpyDeviceToHost, s->stream),
             "read |W|");
+    const StreamWait wait{s->stream};   // on every return from here on
     if (lm_status st = enqueue_lanczos_iteration(s, 0, n, V, w, scal, red, cb, s->lz_ev[0])) return st;
     LM_CUDA(cudaEventSynchronize(s->lz_ev[0]), "lanczos");
     const double normW = s->pinned[kScal * (m_max + 2)];
@@ -1279,23 +1287,15 @@ static lm_status sqrt_mdot_body(lm_solver* s, const double* W, uint64_t seed, do
             if (lm_status st = enqueue_lanczos_iteration(s, k + 1, n, V, w, scal, red, cb, s->lz_ev[k + 1])) return st;
         }
         LM_CUDA(cudaEventSynchronize(s->lz_ev[k]), "lanczos iteration");
-        if (s->lz_one && s->pinned[kScal * k + 3] != 0.0) {
-            cudaStreamSynchronize(s->stream);   // the iteration that runs ahead still writes s->pinned
-            return fail(LM_ERR_TIMEOUT, "a device-side wait expired");
-        }
+        if (s->lz_one && s->pinned[kScal * k + 3] != 0.0) return fail(LM_ERR_TIMEOUT, "a device-side wait expired");
         const double a_k = s->pinned[kScal * k];
         const double b_k = s->pinned[kScal * k + 1];
-        if (!std::isfinite(a_k) || !std::isfinite(b_k)) {
-            cudaStreamSynchronize(s->stream);
+        if (!std::isfinite(a_k) || !std::isfinite(b_k))
             return fail(LM_ERR_CUDA, "Lanczos produced a non-finite coefficient at iteration %d", k + 1);
-        }
         H.alpha.push_back(a_k);
         const int m = k + 1;
         int ncl = 0;
-        if (H.solve(m, normW, &ncl) != 0) {
-            cudaStreamSynchronize(s->stream);
-            return fail(LM_ERR_NOT_CONVERGED, "tridiagonal eigensolver did not converge");
-        }
+        if (H.solve(m, normW, &ncl) != 0) return fail(LM_ERR_NOT_CONVERGED, "tridiagonal eigensolver did not converge");
         clamped = ncl;
         bool stop = false;
         if (k >= 1) {

@@ -1,7 +1,7 @@
 """The one-launch Lanczos iteration when its launch is refused (the separate
-kernels serve) and when a wait among its CTAs runs out (LM_ERR_TIMEOUT, and the
-solver stays usable), in the bounds-checked build, which can be told to make
-either happen."""
+kernels serve; LM_ERR_CUDA when that happens with an iteration in flight) and
+when a wait among its CTAs runs out (LM_ERR_TIMEOUT), in the bounds-checked
+build, which can be told to make each happen.  The solver stays usable."""
 import os
 import subprocess
 import sys
@@ -30,13 +30,20 @@ for n, fp64 in ((1, False), (700, False), (700, True), (5000, False)):
     z = root()
     # each within 20 tol of the root
     assert float((y - z).norm() / y.norm()) <= 40 * tol, n
-    if n == 700:
-        os.environ["LM_DEBUG_LANCZOS_STEP"] = "expire"
+    for fault, status in (("refuse_later", lm.LM_ERR_CUDA), ("expire", lm.LM_ERR_TIMEOUT)):
+        if n != 700:
+            continue
+        os.environ["LM_DEBUG_LANCZOS_STEP"] = fault
         try:
             root()
-            raise SystemExit("no timeout")
+            raise SystemExit("no error from " + fault)
         except lm.LmError as e:
-            assert e.status == lm.LM_ERR_TIMEOUT, e
+            assert e.status == status, e
+        # the scalars' memory grows for more iterations, and the flag of the next positions lies in it
+        del os.environ["LM_DEBUG_LANCZOS_STEP"]
+        lm.lm_sqrt_mdot(s, W, tol=tol, max_iter=100 + 50 * status)
+        lm.lm_set_positions(s, torch.from_numpy(s_.pos).cuda())
+        os.environ["LM_DEBUG_LANCZOS_STEP"] = "none"
     del os.environ["LM_DEBUG_LANCZOS_STEP"]
     assert torch.equal(y, root()), n
 lm.lm_debug_check()
