@@ -52,12 +52,13 @@ FP32_LANES_PER_SM = 128
 RECIPE_MAX_SM_MHZ = 2070.0
 FLOPS_PER_PAIR_TT = 35   # translation-only far-field pair, one-sided (the batched workload)
 # ncu summaries of the product's kernel (DRAM bytes per launch), per workload and form (symmetric or one-sided)
-PAIR_PROFILE = {("melt", False): "pair_kernel_melt_n524288.txt", ("rpy6", True): "sym_kernel_rpy6_n32768.txt"}
+PAIR_PROFILE = {("melt", False): "pair_kernel_melt_n524288.txt", ("rpy6", False): "pair_kernel_rpy6_n32768.txt",
+                ("rpy6", True): "sym_kernel_rpy6_n32768.txt"}
 PAIR_KERNEL_SRCS = {False: ("pair_kernels.cu", "pair_common.cuh"),
                     True: ("sym_kernels.cu", "sym_common.cuh", "pair_common.cuh")}
 
 
-def pair_kernel_source_hash(symmetric: bool) -> str:
+def pair_kernel_source_hash(symmetric: bool = False) -> str:
     h = hashlib.sha256()
     for f in PAIR_KERNEL_SRCS[symmetric]:
         h.update(open(os.path.join(ROOT, "paper_2510_02135_gb300", "csrc", f), "rb").read())
@@ -148,7 +149,7 @@ def measured_hbm_gbs():
         return 6800.0
 
 
-def profile_traffic(workload: str, symmetric: bool):
+def profile_traffic(workload: str, symmetric: bool = False):
     """DRAM bytes per launch of the product's kernel from the committed ncu
     summary of this workload and form, if it was taken on the current kernel
     source (else None)."""
